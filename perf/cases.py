@@ -88,6 +88,8 @@ def draw(rng):
                 break
         prec = rng.choice(["f32", "f32", "f16", "f64"])
         nrhs = min(_log_int(rng, 1, 12), max(1, 4 * 24 ** 3 * 48 // math.prod(dims)))
+        if prec == "f16" and math.prod(dims) % 4:
+            nrhs = 1   # a half-precision field of such a volume does not end on a 16-byte boundary
         if prec == "f64":
             nrhs = min(nrhs, max(1, 16 ** 3 * 32 * 4 // math.prod(dims)))
         return dict(kind=kind, lx=dims[0], ly=dims[1], lz=dims[2], lt=dims[3], prec=prec, nrhs=nrhs, eps=eps,
