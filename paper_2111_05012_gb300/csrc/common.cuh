@@ -320,7 +320,11 @@ template <> struct SpinorIO<P16> {
     }
 };
 
-template <class P> HD size_t spinor_bytes(int V) { return SpinorIO<P>::bytes_per_site * (size_t)V; }
+// bytes from one field of a batch to the next: whole 16-byte words (52 V bytes of a half field are
+// not, unless V is a multiple of four, and the next field's 16-byte accesses would be misaligned)
+template <class P> HD size_t spinor_bytes(int V) {
+    return (SpinorIO<P>::bytes_per_site * (size_t)V + 15) / 16 * 16;
+}
 
 // ---------------------------------------------------------------- gauge storage
 //   P64: [mu][9][V] double2 (full matrix, row-major)
