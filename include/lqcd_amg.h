@@ -270,7 +270,8 @@ amg_status amg_apply_D_noalloc(amg_dirac* d, const void* in, void* out, int nrhs
  * the register budget (2 resident CTAs per SM, 128 registers, against the
  * default).  The choice is process-wide and used by every later stencil
  * launch of that precision (amg_setup runs the same tuner for the precisions
- * a solve uses).  Outputs (may be NULL): threads per CTA, grid cap in CTAs
+ * a solve uses); amg_apply_D on 16-byte aligned vectors runs a kernel of its own
+ * on the canonical layout, in a fixed shape.  Outputs (may be NULL): threads per CTA, grid cap in CTAs
  * per SM, register budget as resident CTAs per SM (0 = the default).
  * Synchronises the device.  No counterpart in the paper. */
 amg_status amg_dirac_tune(amg_dirac* d, amg_prec prec, int* threads, int* per_sm, int* regs_ctas);

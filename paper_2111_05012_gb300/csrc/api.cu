@@ -2550,7 +2550,22 @@ static amg_status apply_fine_canonical(amg_dirac* d, const BlockH* sb, const voi
     }
     if (prec < 0 || prec > 2)
         return fail(AMG_EINVAL, "prec must be AMG_F64, AMG_F32, AMG_F16 (or AMG_F64X / AMG_F64D for D)");
-    size_t fb = fine_spinor_bytes(prec, g.V) * nrhs;
+    const size_t fb = fine_spinor_bytes(prec, g.V) * nrhs;
+    // one pass over the caller's vectors where the kernel can read and write them as they are:
+    // aligned to 16 bytes and apart from each other (overlapping vectors go through the work
+    // fields below, where the input is copied before the output is written)
+    const size_t cb = (size_t)g.V * 24 * (prec == AMG_F64 ? sizeof(double) : sizeof(float)) * nrhs;
+    const bool apart = (const char*)in + cb <= (const char*)out || (const char*)out + cb <= (const char*)in;
+    if (apart && dirac_canon_supported(in, out)) {
+        const void* src = in;
+        if (prec == AMG_F16) {   // rounded to half precision once per site
+            CK(d->in.ensure(fb));
+            CK(launch_pack_spinor(prec, g, in, d->in.p, nrhs, s));
+            src = d->in.p;
+        }
+        CK(launch_dirac_canon(prec, g, sb, d->gauge->U[prec].p, d->C[prec].p, src, out, d->kappa, nrhs, s));
+        return AMG_OK;
+    }
     CK(d->in.ensure(fb));
     CK(d->out.ensure(fb));
     CK(launch_pack_spinor(prec, g, in, d->in.p, nrhs, s));

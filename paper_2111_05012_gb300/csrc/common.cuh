@@ -318,6 +318,18 @@ template <> struct SpinorIO<P16> {
         }
         scale[s] = m;
     }
+    // the values a store followed by a load gives back, in registers
+    DEV static void round_to_storage(cx<float> v[12]) {
+        float m = 0.f;
+#pragma unroll
+        for (int k = 0; k < 12; ++k) m = fmaxf(m, fmaxf(fabsf(v[k].re), fabsf(v[k].im)));
+        const float inv = m > 0.f ? 1.f / m : 0.f;
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            const float2 f = __half22float2(__floats2half2_rn(v[k].re * inv, v[k].im * inv));
+            v[k] = {f.x * m, f.y * m};
+        }
+    }
 };
 
 // bytes from one field of a batch to the next: whole 16-byte words (52 V bytes of a half field are
@@ -564,6 +576,35 @@ template <typename T> DEV T warp_sum(T v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
+}
+
+// Warp sums of N values per lane (N a power of two, N <= 32) with 2N - 1 + log2(32/N)
+// shuffles instead of 5N: each halving step pairs lanes l and l^off, every lane keeping
+// one half of its values (the lower half if its bit off is clear) plus the partner's
+// copy of that half.  Afterwards lane l holds the total of value sum_t bit(l, 4-t) * N/2^(t+1)
+// (see transposed_index), duplicated over the lanes that differ only in the low bits.
+template <int N, typename T> DEV T transposed_warp_sum(T (&v)[N], int lane) {
+#pragma unroll
+    for (int t = 0, h = N / 2, off = 16; h >= 1; ++t, h /= 2, off /= 2) {
+        const bool up = (lane & off) != 0;
+#pragma unroll
+        for (int k = 0; k < h; ++k) {
+            const T keep = up ? v[k + h] : v[k];
+            const T give = up ? v[k] : v[k + h];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, give, off);
+        }
+    }
+    T r = v[0];
+#pragma unroll
+    for (int off = 16 / N; off >= 1; off /= 2) r += __shfl_xor_sync(0xffffffffu, r, off);
+    return r;
+}
+template <int N> DEV int transposed_index(int lane) {
+    int idx = 0;
+#pragma unroll
+    for (int t = 0, h = N / 2, off = 16; h >= 1; ++t, h /= 2, off /= 2)
+        if (lane & off) idx += h;
+    return idx;
 }
 
 // Sum of NV values over the whole block; every thread gets the totals.

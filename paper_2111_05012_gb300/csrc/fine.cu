@@ -2,6 +2,7 @@
 // Wilson-clover stencil of Eq. 1 (full and domain-decomposed D_SAP) and the
 // fused SAP half sweep (Sec. 3, SAP listing with minimal-residual domain
 // solves).
+#include <algorithm>
 #include <cstring>
 
 #include "common.cuh"
@@ -393,54 +394,142 @@ __global__ void clover_expand_kernel(Geom g, const void* C64, double* out) {
 // ------------------------------------------------------------ Wilson-clover stencil
 // FP32 / FP16: three CTAs per SM (the stencil streams from HBM and needs the
 // warps); FP64: two (register cap 128)
+template <class P, bool SAP, class SRC>
+DEV void dirac_sum(const Geom& g, const Blocking& bk, const void* __restrict__ U, const void* __restrict__ C,
+                   const char* src, typename P::T kappa, int s, cx<typename P::T> (&acc)[12]) {
+    using T = typename P::T;
+    int c[4];
+    site_coords(g, s, c);
+    cx<T> psi[12];
+    SRC::load(src, g.V, s, psi);
+    clover_apply<P>(C, g.V, s, psi, acc);
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) {
+        float ph;
+        cx<T> u[3][3];
+        if (!SAP || (c[mu] % bk.b[mu]) != bk.b[mu] - 1) {
+            int n = neighbour(g, s, c, mu, +1, ph);
+            SRC::load(src, g.V, n, psi);
+            GaugeIO<P>::load(U, g.V, mu, s, u);
+            hop_accum<T>(acc, psi, u, mu, +1, -kappa * T(ph));
+        }
+        if (!SAP || (c[mu] % bk.b[mu]) != 0) {
+            int n = neighbour(g, s, c, mu, -1, ph);
+            SRC::load(src, g.V, n, psi);
+            GaugeIO<P>::load(U, g.V, mu, n, u);
+            hop_accum<T>(acc, psi, u, mu, -1, -kappa * T(ph));
+        }
+    }
+}
 template <class P, bool SAP, bool RESID>
 DEV void dirac_site(const Geom& g, const Blocking& bk, const void* __restrict__ U, const void* __restrict__ C,
                     const char* src, char* dst, const char* bsrc, typename P::T kappa, int s) {
     using T = typename P::T;
-    {
-        int c[4];
-        site_coords(g, s, c);
-        cx<T> psi[12], acc[12];
-        SpinorIO<P>::load(src, g.V, s, psi);
-        clover_apply<P>(C, g.V, s, psi, acc);
+    cx<T> acc[12];
+    dirac_sum<P, SAP, SpinorIO<P>>(g, bk, U, C, src, kappa, s, acc);
+    if (RESID) {
+        cx<T> psi[12];
+        SpinorIO<P>::load(bsrc, g.V, s, psi);
 #pragma unroll
-        for (int mu = 0; mu < 4; ++mu) {
-            float ph;
-            cx<T> u[3][3];
-            if (!SAP || (c[mu] % bk.b[mu]) != bk.b[mu] - 1) {
-                int n = neighbour(g, s, c, mu, +1, ph);
-                SpinorIO<P>::load(src, g.V, n, psi);
-                GaugeIO<P>::load(U, g.V, mu, s, u);
-                hop_accum<T>(acc, psi, u, mu, +1, -kappa * T(ph));
-            }
-            if (!SAP || (c[mu] % bk.b[mu]) != 0) {
-                int n = neighbour(g, s, c, mu, -1, ph);
-                SpinorIO<P>::load(src, g.V, n, psi);
-                GaugeIO<P>::load(U, g.V, mu, n, u);
-                hop_accum<T>(acc, psi, u, mu, -1, -kappa * T(ph));
-            }
-        }
-        if (RESID) {
-            SpinorIO<P>::load(bsrc, g.V, s, psi);
-#pragma unroll
-            for (int k = 0; k < 12; ++k) acc[k] = psi[k] - acc[k];
-        }
-        SpinorIO<P>::store(dst, g.V, s, acc);
+        for (int k = 0; k < 12; ++k) acc[k] = psi[k] - acc[k];
     }
+    SpinorIO<P>::store(dst, g.V, s, acc);
 }
 // MB: resident CTAs per SM the register budget is set for (launch bounds; 0 = the default of
-// the precision); the autotuner picks it with the CTA size and grid cap
+// the precision); the autotuner picks it with the CTA size and grid cap.  The right-hand side is
+// the fast grid index: the CTAs of one stretch of sites for all right-hand sides run together
+// and read its links and clover from L2 instead of from DRAM once per right-hand side.
 template <class P, bool SAP, bool RESID, int MB = 0>
 __global__ void __launch_bounds__(kThreads, MB ? MB : (P::id == 0 ? 2 : 3)) dirac_kernel(Geom g, Blocking bk, const void* __restrict__ U,
                                                          const void* __restrict__ C, const void* in, void* out,
                                                          const void* b, typename P::T kappa) {
-    const int r = blockIdx.y;
+    const int r = blockIdx.x;
     const size_t fb = spinor_bytes<P>(g.V);
     const char* src = (const char*)in + r * fb;
     char* dst = (char*)out + r * fb;
     const char* bsrc = RESID ? (const char*)b + r * fb : nullptr;
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < g.V; s += gridDim.x * blockDim.x)
+    for (int s = blockIdx.y * blockDim.x + threadIdx.x; s < g.V; s += gridDim.y * blockDim.x)
         dirac_site<P, SAP, RESID>(g, bk, U, C, src, dst, bsrc, kappa, s);
+}
+
+// The same stencil on the caller's canonical vectors (24 values per site, one site after
+// another), without a pass to the internal layout and back.
+// CIN: read the canonical input as it is (FP32, FP64); else the internal field (FP16, whose
+// values are rounded once per site by pack, not once per neighbour).  A site's record is six
+// (FP32) or twelve (FP64) consecutive 16-byte words, so a warp's six loads together use every
+// byte of the lines they touch.
+// The result goes out through a shared-memory tile of the warp (25 words per site, so that the
+// per-site writes fall in different banks) as consecutive 16-byte words; FP64, bound by the FP64
+// pipe, stores its records directly.
+template <class P> struct CanonIn;
+template <> struct CanonIn<P32> {
+    DEV static void load(const void* base, int, int s, cx<float> v[12]) {
+        const float4* p = (const float4*)base + (size_t)s * 6;
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+            const float4 t = __ldg(p + c);
+            v[2 * c] = {t.x, t.y};
+            v[2 * c + 1] = {t.z, t.w};
+        }
+    }
+};
+template <> struct CanonIn<P64> {
+    DEV static void load(const void* base, int, int s, cx<double> v[12]) {
+        const double2* p = (const double2*)base + (size_t)s * 12;
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            const double2 t = __ldg(p + k);
+            v[k] = {t.x, t.y};
+        }
+    }
+};
+template <> struct CanonIn<P16> : SpinorIO<P16> {};
+
+// 128 threads at 128 registers: with the three-CTA budget of dirac_kernel (80 registers) FP32
+// spills 268 bytes a thread (346 us at 32^3 x 64 against 263 us), and 128 threads leave a
+// shorter last wave than 256 (FP64, 16^3 x 32: 269 us against 305 us).  FP32 at 32^3 x 64 is
+// bound by HBM and by the L1's handling of records (1.41 GB, 207 us at 6.8 TB/s); with the two
+// layout passes it replaces the call took 391 us.  FP16, 24^3 x 48, four right-hand sides:
+// 386 -> 283 us (pack 54 us of it); FP64, 16^3 x 32: 326 -> 269 us, the FP64 pipe's time.
+constexpr int kCanonThreads = 128;
+template <class P, bool SAP>
+__global__ void __launch_bounds__(kCanonThreads, 4)
+    dirac_canon_kernel(Geom g, Blocking bk, const void* __restrict__ U, const void* __restrict__ C,
+                       const void* __restrict__ in, void* __restrict__ out, typename P::T kappa) {
+    using T = typename P::T;
+    extern __shared__ __align__(16) float canon_tile[];   // [warps][32 * kPad], FP32 and FP16
+    const int r = blockIdx.x, lane = threadIdx.x & 31;
+    const char* src = (const char*)in + r * (P::id == 2 ? spinor_bytes<P>(g.V) : (size_t)g.V * 24 * sizeof(T));
+    T* dst = (T*)out + (size_t)r * g.V * 24;
+    // the loop is uniform over a warp: s0 is the warp's first site
+    for (int s0 = blockIdx.y * blockDim.x + (threadIdx.x & ~31); s0 < g.V; s0 += gridDim.y * blockDim.x) {
+        const int s = s0 + lane;
+        cx<T> acc[12];
+        if (s < g.V) dirac_sum<P, SAP, CanonIn<P>>(g, bk, U, C, src, kappa, s, acc);
+        if constexpr (P::id == 0) {
+            if (s < g.V) {
+                double2* o = (double2*)dst + (size_t)s * 12;
+#pragma unroll
+                for (int k = 0; k < 12; ++k) o[k] = make_double2(acc[k].re, acc[k].im);
+            }
+        } else {
+            float* w = canon_tile + (threadIdx.x >> 5) * 32 * kPad;
+            if (s < g.V) {
+                if constexpr (P::id == 2) SpinorIO<P16>::round_to_storage(acc);
+                float* e = w + lane * kPad;
+#pragma unroll
+                for (int k = 0; k < 12; ++k) {
+                    e[2 * k] = acc[k].re;
+                    e[2 * k + 1] = acc[k].im;
+                }
+            }
+            __syncwarp();
+            const int nv = min(32, g.V - s0) * 6;   // 16-byte words of the warp's sites
+            float4* o = (float4*)(dst + (size_t)s0 * 24);
+            for (int i = lane; i < nv; i += 32) o[i] = Vec16<float>::make(w + tile_pos(4 * i));
+            __syncwarp();
+        }
+    }
 }
 
 // ragged batch, restart phases (site loops over each problem's lattice)
@@ -1661,6 +1750,12 @@ struct DiracShape {
 };
 DiracShape g_dirac_shape[3] = {{kThreads, 16, 0}, {kThreads, 16, 0}, {kThreads, 16, 0}};
 
+// right-hand side x stretch of sites, the stretches capped at per_sm CTAs per SM (grid-stride loop)
+dim3 dirac_grid(int V, int threads, int per_sm, int nrhs) {
+    const long long cap = std::min<long long>((long long)device_sms() * per_sm, 65535);
+    return dim3(nrhs, (unsigned)std::min<long long>((V + threads - 1) / threads, cap));
+}
+
 template <class P>
 cudaError_t dirac_impl(const GeomH& gh, const BlockH* sb, const void* U, const void* C, const void* in, void* out,
                        const void* b, double kappa, int nrhs, cudaStream_t st) {
@@ -1669,10 +1764,7 @@ cudaError_t dirac_impl(const GeomH& gh, const BlockH* sb, const void* U, const v
     BlockH one = {{1, 1, 1, 1}};
     bk = make_blocking(gh, sb ? *sb : one);
     const DiracShape sh = g_dirac_shape[P::id];
-    int blocks = (g.V + sh.threads - 1) / sh.threads;
-    const int cap = device_sms() * sh.per_sm;
-    if (blocks > cap) blocks = cap;
-    dim3 grid(blocks, nrhs);
+    const dim3 grid = dirac_grid(g.V, sh.threads, sh.per_sm, nrhs);
     const int th = sh.threads;
     using T = typename P::T;
     if (sb) {
@@ -1689,6 +1781,24 @@ cudaError_t dirac_impl(const GeomH& gh, const BlockH* sb, const void* U, const v
     }
     if (b) (note_launch(), dirac_kernel<P, false, true><<<grid, th, 0, st>>>(g, bk, U, C, in, out, b, (T)kappa));
     else (note_launch(), dirac_kernel<P, false, false><<<grid, th, 0, st>>>(g, bk, U, C, in, out, b, (T)kappa));
+    return cudaGetLastError();
+}
+
+template <class P>
+cudaError_t dirac_canon_impl(const GeomH& gh, const BlockH* sb, const void* U, const void* C, const void* in,
+                             void* out, double kappa, int nrhs, cudaStream_t st) {
+    Geom g = make_geom(gh);
+    const BlockH one = {{1, 1, 1, 1}};
+    const Blocking bk = make_blocking(gh, sb ? *sb : one);
+    // a lattice with less than a full CTA per SM is spread over more, smaller CTAs (4^4: one
+    // launch of 6.2 us against 14.3 us for the three it replaces)
+    int th = kCanonThreads;
+    while (th > 32 && (long long)g.V * nrhs < (long long)device_sms() * th) th /= 2;
+    const dim3 grid = dirac_grid(g.V, th, 65535, nrhs);
+    const size_t smem = P::id == 0 ? 0 : (size_t)th * kPad * sizeof(float);
+    using T = typename P::T;
+    if (sb) (note_launch(), dirac_canon_kernel<P, true><<<grid, th, smem, st>>>(g, bk, U, C, in, out, (T)kappa));
+    else (note_launch(), dirac_canon_kernel<P, false><<<grid, th, smem, st>>>(g, bk, U, C, in, out, (T)kappa));
     return cudaGetLastError();
 }
 
@@ -1852,6 +1962,15 @@ cudaError_t launch_dirac(int prec, const GeomH& g, const BlockH* sb, const void*
     if (prec == 0) return dirac_impl<P64>(g, sb, U, C, in, out, b, kappa, nrhs, st);
     if (prec == 1) return dirac_impl<P32>(g, sb, U, C, in, out, b, kappa, nrhs, st);
     return dirac_impl<P16>(g, sb, U, C, in, out, b, kappa, nrhs, st);
+}
+bool dirac_canon_supported(const void* in, const void* out) {
+    return (((uintptr_t)in | (uintptr_t)out) & 15) == 0;
+}
+cudaError_t launch_dirac_canon(int prec, const GeomH& g, const BlockH* sb, const void* U, const void* C,
+                               const void* in, void* out, double kappa, int nrhs, cudaStream_t st) {
+    if (prec == 0) return dirac_canon_impl<P64>(g, sb, U, C, in, out, kappa, nrhs, st);
+    if (prec == 1) return dirac_canon_impl<P32>(g, sb, U, C, in, out, kappa, nrhs, st);
+    return dirac_canon_impl<P16>(g, sb, U, C, in, out, kappa, nrhs, st);
 }
 cudaError_t launch_dirac_mixed(const GeomH& gh, const void* Udd, const void* Cdd, const void* in32, void* out64,
                                double kappa, int nrhs, cudaStream_t st) {

@@ -55,6 +55,12 @@ void dirac_get_shape(int prec, int* threads, int* per_sm, int* mb = nullptr);
 // out = D in (sap_block != NULL: hops between blocks removed); if b != NULL, out = b - D in
 cudaError_t launch_dirac(int prec, const GeomH& g, const BlockH* sap_block, const void* U, const void* C,
                          const void* in, void* out, const void* b, double kappa, int nrhs, cudaStream_t s);
+// The same D on canonical vectors (no residual form): in is canonical for FP64 and FP32, the
+// internal field for FP16; out is canonical.  Both 16-byte aligned (dirac_canon_supported), not
+// overlapping.
+bool dirac_canon_supported(const void* in, const void* out);
+cudaError_t launch_dirac_canon(int prec, const GeomH& g, const BlockH* sap_block, const void* U, const void* C,
+                               const void* in, void* out, double kappa, int nrhs, cudaStream_t s);
 // out (FP64 internal) = D in (FP32 internal, exact values) with FP64-accurate double-float arithmetic;
 // Udd / Cdd are the prec-3 (float hi/lo pair) link and clover fields
 cudaError_t launch_dirac_mixed(const GeomH& g, const void* Udd, const void* Cdd, const void* in32, void* out64,

@@ -94,35 +94,6 @@ template <> struct RawSite<P16> {   // three uint4 of halves, then the per-site 
 // vectors whose loads a thread keeps in flight together
 template <class PV> constexpr int kVecGroup = PV::id == 2 ? 4 : 2;
 
-// Warp sums of N values per lane (N a power of two, N <= 32) with 2N - 1 + log2(32/N)
-// shuffles instead of 5N: each halving step pairs lanes l and l^off, every lane keeping
-// one half of its values (the lower half if its bit off is clear) plus the partner's
-// copy of that half.  Afterwards lane l holds the total of value sum_t bit(l, 4-t) * N/2^(t+1)
-// (see transposed_index), duplicated over the lanes that differ only in the low bits.
-template <int N, typename T> DEV T transposed_warp_sum(T (&v)[N], int lane) {
-#pragma unroll
-    for (int t = 0, h = N / 2, off = 16; h >= 1; ++t, h /= 2, off /= 2) {
-        const bool up = (lane & off) != 0;
-#pragma unroll
-        for (int k = 0; k < h; ++k) {
-            const T keep = up ? v[k + h] : v[k];
-            const T give = up ? v[k] : v[k + h];
-            v[k] = keep + __shfl_xor_sync(0xffffffffu, give, off);
-        }
-    }
-    T r = v[0];
-#pragma unroll
-    for (int off = 16 / N; off >= 1; off /= 2) r += __shfl_xor_sync(0xffffffffu, r, off);
-    return r;
-}
-template <int N> DEV int transposed_index(int lane) {
-    int idx = 0;
-#pragma unroll
-    for (int t = 0, h = N / 2, off = 16; h >= 1; ++t, h /= 2, off /= 2)
-        if (lane & off) idx += h;
-    return idx;
-}
-
 // ------------------------------------------------------------ restriction
 // One CTA per block, one thread per site: the site's share of <X,s,i|psi> for a
 // group of test vectors (their loads in flight together), summed over the warp
