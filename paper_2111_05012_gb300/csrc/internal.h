@@ -60,13 +60,11 @@ struct amg_nn {
     DevBuf wadj[AMG_NN_MAX_LAYERS];         // bfloat16 adjoint weights (input gradient)
     DevBuf act[AMG_NN_MAX_LAYERS + 1];      // activations, FP32 internal fields x channels
     DevBuf gbuf[2];                         // gradient fields
-    DevBuf ework;                           // target field
+    DevBuf ework;                           // output field
     DevBuf part;                            // reduction partials
-    DevBuf canon;                           // canonical staging
-    double* hpart = nullptr;                // pinned partials
-    ~amg_nn() {
-        if (hpart) cudaFreeHost(hpart);
-    }
+    DevBuf grad[AMG_NN_MAX_LAYERS];         // weight gradients, summed over a batch's pairs
+    DevBuf norms;                           // per pair (|y - e|^2, |e|^2)
+    DevBuf ecopy;                           // aligned copy of an unaligned target batch
 };
 
 // accessors implemented in api.cu
@@ -76,12 +74,15 @@ const void* amg_internal_links(const amg_dirac* d, int prec);
 void amg_internal_set_error(const char* msg);
 
 // PT-conv launchers (ptconv.cu)
-int ptconv_grid();
+size_t ptconv_partials(int cin, int cout);   // double2 entries of part for a layer
+// out = layer(in).  With target (one output channel, canonical floats): out = layer(in) - target,
+// and *norms = (|out|^2, |target|^2), through the CTAs' shares in part.
 cudaError_t launch_ptconv_forward(const GeomH& g, int cin, int cout, const void* U32, const void* Wbf16,
-                                  const void* in, void* out, cudaStream_t s);
+                                  const void* in, void* out, cudaStream_t s, const float* target = nullptr,
+                                  double2* part = nullptr, double2* norms = nullptr);
+// G (+)= the layer's weight gradient [cout][cin][9][4][4] (device), over norm->y if norm is given
 cudaError_t launch_ptconv_wgrad(const GeomH& g, int cin, int cout, const void* U32, const void* in, const void* gout,
-                                double2* part, cudaStream_t s);
-cudaError_t launch_residual_scale(void* y, const void* e, size_t n, float scale, double* part, cudaStream_t s);
+                                double2* part, const double2* norm, bool add, double2* G, cudaStream_t s);
 
 // network forward on FP32 internal fields: out = N(in) (nn_api.cu)
 amg_status nn_forward_internal(amg_nn* nn, const void* in32, void* out32, cudaStream_t s);

@@ -1,6 +1,7 @@
 // C ABI of the learned parallel-transport preconditioner: creation, weights,
 // single-layer forward / backward (for parity tests), one Adam training step
 // on a batch of (residual, error) pairs.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -73,33 +74,10 @@ amg_status upload_weights(amg_nn* nn) {
 const GeomH& geom(amg_nn* nn) { return *amg_internal_geom(nn->d); }
 size_t fbytes(amg_nn* nn) { return fine_spinor_bytes(1, geom(nn).V); }
 
-amg_status sum_partials(amg_nn* nn, size_t count, double* out, cudaStream_t s) {
-    NCK(cudaMemcpyAsync(nn->hpart, nn->part.p, count * sizeof(double), cudaMemcpyDeviceToHost, s));
+// the layer's gradient on the device as host doubles (waits for the stream)
+amg_status fetch_grad(amg_nn* nn, int l, double* out, cudaStream_t s) {
+    NCK(cudaMemcpyAsync(out, nn->grad[l].p, layer_size(nn, l) * sizeof(double), cudaMemcpyDeviceToHost, s));
     NCK(cudaStreamSynchronize(s));
-    for (size_t i = 0; i < count; ++i) out[i] = nn->hpart[i];
-    return AMG_OK;
-}
-
-// weight gradient of layer l (Wirtinger, [cout][cin][9][4][4][re,im]) from the
-// layer input field (cin channels) and the output gradient (cout channels)
-amg_status layer_wgrad(amg_nn* nn, int l, const void* in, const void* gout, std::vector<double>& G, cudaStream_t s) {
-    const int cin = nn->ch[l], cout = nn->ch[l + 1];
-    const int grid = ptconv_grid();
-    const size_t per = (size_t)cout * 16;   // complex per CTA per (b, d)
-    NCK(launch_ptconv_wgrad(geom(nn), cin, cout, amg_internal_links(nn->d, 1), in, gout, nn->part.as<double2>(), s));
-    std::vector<double> h((size_t)cin * 9 * grid * per * 2);
-    NTRY(sum_partials(nn, h.size(), h.data(), s));
-    G.assign(layer_size(nn, l), 0.0);
-    for (int b = 0; b < cin; ++b)
-        for (int d = 0; d < 9; ++d)
-            for (int blk = 0; blk < grid; ++blk)
-                for (int a = 0; a < cout; ++a)
-                    for (int k = 0; k < 16; ++k) {
-                        const size_t src = ((((size_t)(b * 9 + d) * grid + blk) * per) + a * 16 + k) * 2;
-                        const size_t dst = ((((size_t)a * cin + b) * 9 + d) * 16 + k) * 2;
-                        G[dst] += h[src];
-                        G[dst + 1] += h[src + 1];
-                    }
     return AMG_OK;
 }
 
@@ -111,14 +89,12 @@ amg_status ensure_buffers(amg_nn* nn) {
     NCK(nn->gbuf[0].ensure(fb * cmax));
     NCK(nn->gbuf[1].ensure(fb * cmax));
     NCK(nn->ework.ensure(fb));
-    size_t pmax = 4096;
+    size_t pmax = 0;
     for (int l = 0; l < nn->nlayers; ++l) {
-        size_t q = (size_t)nn->ch[l] * 9 * ptconv_grid() * nn->ch[l + 1] * 16 * 2;
-        pmax = q > pmax ? q : pmax;
+        pmax = std::max(pmax, ptconv_partials(nn->ch[l], nn->ch[l + 1]));
+        NCK(nn->grad[l].ensure(layer_size(nn, l) * sizeof(double)));
     }
-    NCK(nn->part.ensure(pmax * sizeof(double)));
-    if (!nn->hpart) NCK(cudaMallocHost(&nn->hpart, pmax * sizeof(double)));
-    NCK(nn->canon.ensure((size_t)geom(nn).V * 24 * sizeof(float) * cmax));
+    NCK(nn->part.ensure(pmax * sizeof(double2)));
     return AMG_OK;
 }
 
@@ -199,9 +175,9 @@ amg_status amg_nn_layer_backward(amg_nn* nn, int layer, const float* in, const f
     NCK(launch_pack_spinor(1, g, in, nn->gbuf[0].p, cin, s));
     NCK(launch_pack_spinor(1, g, grad_out, nn->gbuf[1].p, cout, s));
     if (grad_w) {
-        std::vector<double> G;
-        NTRY(layer_wgrad(nn, layer, nn->gbuf[0].p, nn->gbuf[1].p, G, s));
-        std::memcpy(grad_w, G.data(), G.size() * sizeof(double));
+        NCK(launch_ptconv_wgrad(g, cin, cout, amg_internal_links(nn->d, 1), nn->gbuf[0].p, nn->gbuf[1].p,
+                                nn->part.as<double2>(), nullptr, false, nn->grad[layer].as<double2>(), s));
+        NTRY(fetch_grad(nn, layer, grad_w, s));
     }
     if (grad_in) {
         NCK(launch_ptconv_forward(g, cout, cin, amg_internal_links(nn->d, 1), nn->wadj[layer].p, nn->gbuf[1].p,
@@ -227,43 +203,29 @@ amg_status amg_nn_train_step(amg_nn* nn, const float* r, const float* e, int npa
     if (!nn || !r || !e || npairs < 1 || !(lr > 0)) return nfail(AMG_EINVAL, "bad argument");
     cudaStream_t s = (cudaStream_t)stream;
     const GeomH& g = geom(nn);
-    const size_t n = (size_t)g.V * 12;   // complex numbers per field
     const int L = nn->nlayers;
-    std::vector<std::vector<double>> gsum(L);
-    for (int l = 0; l < L; ++l) gsum[l].assign(layer_size(nn, l), 0.0);
-    double loss = 0;
+    if (((uintptr_t)e & 15) != 0) {
+        // the loss reads e in 16-byte words: an unaligned batch goes through an aligned copy
+        const size_t bytes = (size_t)npairs * g.V * 24 * sizeof(float);
+        NCK(nn->ecopy.ensure(bytes));
+        NCK(cudaMemcpyAsync(nn->ecopy.p, e, bytes, cudaMemcpyDeviceToDevice, s));
+        e = nn->ecopy.as<float>();
+    }
+    NCK(nn->norms.ensure(npairs * sizeof(double2)));
+    // every pair's gradient is summed on the device, scaled by 1 / |e|^2 as it is added; the
+    // host waits once for the whole batch
     for (int p = 0; p < npairs; ++p) {
+        double2* norm = nn->norms.as<double2>() + p;
         NCK(launch_pack_spinor(1, g, r + (size_t)p * g.V * 24, nn->act[0].p, 1, s));
         for (int l = 0; l < L; ++l)
             NCK(launch_ptconv_forward(g, nn->ch[l], nn->ch[l + 1], amg_internal_links(nn->d, 1), nn->wbf[l].p,
-                                      nn->act[l].p, nn->act[l + 1].p, s));
-        NCK(launch_pack_spinor(1, g, e + (size_t)p * g.V * 24, nn->ework.p, 1, s));
-        // ||e||^2 as the residual of a zero field against e
-        double ne2 = 0;
-        {
-            NCK(cudaMemsetAsync(nn->gbuf[0].p, 0, fbytes(nn), s));
-            NCK(launch_residual_scale(nn->gbuf[0].p, nn->ework.p, n, 1.0f, nn->part.as<double>(), s));
-            std::vector<double> h(ptconv_grid());
-            NTRY(sum_partials(nn, h.size(), h.data(), s));
-            for (double x : h) ne2 += x;
-        }
-        if (!(ne2 > 0)) return nfail(AMG_EINVAL, "amg_nn_train_step: zero error vector");
-        // g = (y - e) / ||e||^2 in place of y, and ||y - e||^2
-        NCK(launch_residual_scale(nn->act[L].p, nn->ework.p, n, (float)(1.0 / ne2), nn->part.as<double>(), s));
-        {
-            std::vector<double> h(ptconv_grid());
-            NTRY(sum_partials(nn, h.size(), h.data(), s));
-            double t = 0;
-            for (double x : h) t += x;
-            loss += t / ne2;
-        }
-        if (!std::isfinite(loss)) return nfail(AMG_NAN, "amg_nn_train_step: non-finite loss");
-        const void* gout = nn->act[L].p;
+                                      nn->act[l].p, nn->act[l + 1].p, s, l == L - 1 ? e + (size_t)p * g.V * 24 : nullptr,
+                                      nn->part.as<double2>(), norm));
+        const void* gout = nn->act[L].p;   // y - e
         int gi = 0;
         for (int l = L - 1; l >= 0; --l) {
-            std::vector<double> G;
-            NTRY(layer_wgrad(nn, l, nn->act[l].p, gout, G, s));
-            for (size_t i = 0; i < G.size(); ++i) gsum[l][i] += G[i];
+            NCK(launch_ptconv_wgrad(g, nn->ch[l], nn->ch[l + 1], amg_internal_links(nn->d, 1), nn->act[l].p, gout,
+                                    nn->part.as<double2>(), norm, p > 0, nn->grad[l].as<double2>(), s));
             if (l > 0) {
                 NCK(launch_ptconv_forward(g, nn->ch[l + 1], nn->ch[l], amg_internal_links(nn->d, 1), nn->wadj[l].p,
                                           gout, nn->gbuf[gi].p, s));
@@ -271,6 +233,17 @@ amg_status amg_nn_train_step(amg_nn* nn, const float* r, const float* e, int npa
                 gi ^= 1;
             }
         }
+    }
+    std::vector<std::vector<double>> gsum(L);
+    for (int l = 0; l < L; ++l) gsum[l].resize(layer_size(nn, l));
+    std::vector<double2> norms(npairs);
+    NCK(cudaMemcpyAsync(norms.data(), nn->norms.p, npairs * sizeof(double2), cudaMemcpyDeviceToHost, s));
+    for (int l = 0; l < L; ++l) NTRY(fetch_grad(nn, l, gsum[l].data(), s));
+    double loss = 0;
+    for (const double2& v : norms) {
+        if (!(v.y > 0)) return nfail(AMG_EINVAL, "amg_nn_train_step: zero error vector");
+        loss += v.x / v.y;
+        if (!std::isfinite(loss)) return nfail(AMG_NAN, "amg_nn_train_step: non-finite loss");
     }
     // Adam on the real and imaginary parts; d/d(Re W) = 2 Re G, d/d(Im W) = 2 Im G (mean over pairs)
     const double b1 = 0.9, b2 = 0.999, eps = 1e-8;

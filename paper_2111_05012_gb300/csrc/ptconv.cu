@@ -5,12 +5,13 @@
 // (fermion boundary phase on the t wrap), W_d^{ab} a complex 4x4 spin matrix
 // stored in bfloat16 and applied with FP32 accumulation.  Fields are FP32
 // internal spinors, C channels stored one after another.
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.h"
 
 namespace {
 
-constexpr int kT = 256;
 constexpr int kMaxC = 4;
 
 Geom make_geom(const GeomH& h) {
@@ -35,40 +36,184 @@ int sms() {
     return n;
 }
 
-// (T_d f)(x) for a 12-component FP32 field f (channel base pointer)
-DEV void transport(const Geom& g, const void* U, const void* f, int s, const int c[4], int d, cx<float> out[12]) {
-    if (d == 0) {
-        SpinorIO<P32>::load(f, g.V, s, out);
-        return;
+// y = U v (dir > 0) or U^dag v (dir < 0) on the three colours of each spin
+DEV void colour_mul(const cx<float> u[3][3], int dir, const cx<float> v[12], cx<float> y[12]) {
+    if (dir > 0) {
+#pragma unroll
+        for (int sp = 0; sp < 4; ++sp)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                cx<float> t = u[a][0] * v[3 * sp];
+                cfma(t, u[a][1], v[3 * sp + 1]);
+                cfma(t, u[a][2], v[3 * sp + 2]);
+                y[3 * sp + a] = t;
+            }
+    } else {
+#pragma unroll
+        for (int sp = 0; sp < 4; ++sp)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                cx<float> t = cmulc(u[0][a], v[3 * sp]);
+                cfmac(t, u[1][a], v[3 * sp + 1]);
+                cfmac(t, u[2][a], v[3 * sp + 2]);
+                y[3 * sp + a] = t;
+            }
     }
-    const int mu = (d - 1) & 3, dir = d <= 4 ? 1 : -1;
+}
+
+// What T_d reads at site s, as loaded: the neighbour's spinor, the link (rows 0 and 1) and the
+// boundary phase.  Kept raw so that the next direction's loads can be in flight under the
+// arithmetic of the current one.
+struct HopSite {
+    int n, link;   // neighbour, and the site that holds the link
     float ph;
-    const int n = neighbour(g, s, c, mu, dir, ph);
-    cx<float> v[12], u[3][3];
-    SpinorIO<P32>::load(f, g.V, n, v);
-    GaugeIO<P32>::load(U, g.V, mu, dir > 0 ? s : n, u);
+};
+DEV HopSite hop_site(const Geom& g, int s, const int c[4], int d) {
+    HopSite h = {s, s, 1.f};
+    // the direction is the same in every lane; unrolled so that c stays in registers
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) {
+        if (d == 1 + mu) h.n = neighbour(g, s, c, mu, 1, h.ph);
+        if (d == 5 + mu) h.link = h.n = neighbour(g, s, c, mu, -1, h.ph);
+    }
+    return h;
+}
+struct RawSpinor {
+    float4 r[6];
+    DEV void load(const void* f, int V, int n) {
+#pragma unroll
+        for (int q = 0; q < 6; ++q) r[q] = __ldg((const float4*)f + (size_t)q * V + n);
+    }
+    DEV void get(cx<float> v[12]) const {
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            v[2 * q] = {r[q].x, r[q].y};
+            v[2 * q + 1] = {r[q].z, r[q].w};
+        }
+    }
+};
+struct RawLink {
+    float4 a, b, c;
+    DEV void load(const void* U, int V, int mu, int n) {
+        const float4* p = (const float4*)U + (size_t)mu * 3 * V;
+        a = __ldg(p + n);
+        b = __ldg(p + (size_t)V + n);
+        c = __ldg(p + (size_t)2 * V + n);
+    }
+    DEV void get(float ph, cx<float> u[3][3]) const {
+        u[0][0] = {a.x, a.y};
+        u[0][1] = {a.z, a.w};
+        u[0][2] = {b.x, b.y};
+        u[1][0] = {b.z, b.w};
+        u[1][1] = {c.x, c.y};
+        u[1][2] = {c.z, c.w};
+        reconstruct_row2(u);
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) u[i][k] = ph * u[i][k];
+    }
+};
+struct RawHop {
+    RawSpinor v;
+    RawLink l;
+    float ph;
+    DEV void load(const Geom& g, const void* U, const void* f, int s, const int c[4], int d) {
+        const HopSite h = hop_site(g, s, c, d);
+        ph = h.ph;
+        v.load(f, g.V, h.n);
+        if (d > 0) l.load(U, g.V, (d - 1) & 3, h.link);
+    }
+    // (T_d f)(s)
+    DEV void get(int d, cx<float> out[12]) const {
+        if (d == 0) {
+            v.get(out);
+            return;
+        }
+        cx<float> f[12], u[3][3];
+        v.get(f);
+        l.get(ph, u);
+        colour_mul(u, d <= 4 ? 1 : -1, f, out);
+    }
+};
+
+// acc += w phi for a complex 4x4 spin matrix w in shared memory (two entries per 16-byte read)
+DEV void spin_mac(cx<float> acc[12], const cx<float>* w, const cx<float> phi[12]) {
 #pragma unroll
     for (int sp = 0; sp < 4; ++sp)
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            cx<float> t = czero<float>();
+        for (int t = 0; t < 4; t += 2) {
+            const float4 q = *reinterpret_cast<const float4*>(w + sp * 4 + t);
 #pragma unroll
-            for (int b = 0; b < 3; ++b) t = t + (dir > 0 ? u[a][b] * v[3 * sp + b] : cmulc(u[b][a], v[3 * sp + b]));
-            out[3 * sp + a] = ph * t;
+            for (int col = 0; col < 3; ++col) {
+                cfma(acc[3 * sp + col], cx<float>{q.x, q.y}, phi[3 * t + col]);
+                cfma(acc[3 * sp + col], cx<float>{q.z, q.w}, phi[3 * (t + 1) + col]);
+            }
         }
 }
 
-// out^a = sum_b sum_d W[a][b][d] T_d in^b; weights bf16 [COUT][CIN][9][4][4][2]
-template <int COUT>
-__global__ void __launch_bounds__(kT) ptconv_forward_kernel(Geom g, int cin, const void* __restrict__ U,
-                                                            const __nv_bfloat16* __restrict__ W, const void* in,
-                                                            void* out) {
-    __shared__ cx<float> w[kMaxC * kMaxC * 9 * 16];
-    const int nw = COUT * cin * 9 * 16;
+// |v|^2 as an unevaluated pair of floats: exact products, every rounding error kept, so that
+// the sums carry about 48 bits without the FP64 pipe (1/64 of the FP32 rate)
+DEV void add_square(dfloat& acc, float v) {
+    const float p = __fmul_rn(v, v);
+    const float e = fmaf(v, v, -p);
+    const dfloat t = two_sum(acc.hi, p);
+    acc.hi = t.hi;
+    acc.lo = __fadd_rn(acc.lo, __fadd_rn(t.lo, e));
+}
+
+// The last layer of a training pass: y is replaced by y - e for the canonical target e, and
+// part[cta] receives the CTA's shares of |y - e|^2 and |e|^2
+struct LossArgs {
+    const float4* e;   // canonical, 6 float4 per site; null outside training
+    double2* part;
+};
+DEV void loss_site(const LossArgs& l, int s, cx<float> acc[12], dfloat& d2, dfloat& e2) {
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+        const float4 e = __ldg(l.e + (size_t)s * 6 + q);
+        acc[2 * q] = acc[2 * q] - cx<float>{e.x, e.y};
+        acc[2 * q + 1] = acc[2 * q + 1] - cx<float>{e.z, e.w};
+        add_square(e2, e.x);
+        add_square(e2, e.y);
+        add_square(e2, e.z);
+        add_square(e2, e.w);
+    }
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        add_square(d2, acc[k].re);
+        add_square(d2, acc[k].im);
+    }
+}
+DEV void loss_block(const LossArgs& l, dfloat d2, dfloat e2) {
+    __shared__ double red[2 * 32];
+    double v[2] = {to_double(d2), to_double(e2)};
+    block_sum<double, 2>(v, red);
+    if (threadIdx.x == 0) l.part[blockIdx.x] = make_double2(v[0], v[1]);
+}
+
+// Forward layers.  The colour transport T_d and the spin matrices W_d act on different indices
+// and commute, so the layer transports whichever side has fewer channels:
+// up (cin <= cout): out^a += W_d^{ab} (T_d in^b), cin transports per direction;
+// down (cin > cout): out^a += T_d (sum_b W_d^{ab} in^b), cout transports per direction.
+// Bound by the FP32 pipe (16 cin cout 9 complex spin entries x 3 colours per site, the
+// transports 8 x 36 complex products per transported channel).  128 threads, so that 160
+// registers still leave three CTAs per SM; the loop over the directions stays rolled to keep the
+// body in the instruction cache.  24^3 x 48: 1 -> 4 channels 331 -> 258 us, 4 -> 1 501 -> 321 us (loss included).
+constexpr int kFT = 128;
+DEV void load_weights(cx<float>* w, const __nv_bfloat16* __restrict__ W, int nw) {
     for (int i = threadIdx.x; i < nw; i += blockDim.x)
         w[i] = {__bfloat162float(W[2 * i]), __bfloat162float(W[2 * i + 1])};
     __syncthreads();
+}
+template <int COUT, bool LOSS>
+__global__ void __launch_bounds__(kFT, COUT >= 3 ? 3 : 4) ptconv_up_kernel(Geom g, int cin, const void* __restrict__ U,
+                                                            const __nv_bfloat16* __restrict__ W, const void* in,
+                                                            void* out, LossArgs loss) {
+    __shared__ __align__(16) cx<float> w[COUT * COUT * 9 * 16];   // cin <= COUT
+    load_weights(w, W, COUT * cin * 9 * 16);
     const size_t fb = spinor_bytes<P32>(g.V);
+    dfloat d2, e2;
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < g.V; s += gridDim.x * blockDim.x) {
         int c[4];
         site_coords(g, s, c);
@@ -77,140 +222,288 @@ __global__ void __launch_bounds__(kT) ptconv_forward_kernel(Geom g, int cin, con
         for (int a = 0; a < COUT; ++a)
 #pragma unroll
             for (int k = 0; k < 12; ++k) acc[a][k] = czero<float>();
-        for (int b = 0; b < cin; ++b) {
-            const char* fin = (const char*)in + b * fb;
-            for (int d = 0; d < 9; ++d) {
-                cx<float> phi[12];
-                transport(g, U, fin, s, c, d, phi);
-#pragma unroll
-                for (int a = 0; a < COUT; ++a) {
-                    const cx<float>* wd = w + ((a * cin + b) * 9 + d) * 16;
-#pragma unroll
-                    for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-                        for (int t = 0; t < 4; ++t) {
-                            const cx<float> ws = wd[sp * 4 + t];
-#pragma unroll
-                            for (int col = 0; col < 3; ++col) cfma(acc[a][3 * sp + col], ws, phi[3 * t + col]);
-                        }
-                }
+        RawHop h;
+        h.load(g, U, in, s, c, 0);
+#pragma unroll 1
+        for (int b = 0, d = 0; b < cin;) {
+            cx<float> phi[12];
+            h.get(d, phi);
+            const cx<float>* wd = w + (b * 9 + d) * 16;
+            if (++d == 9) {
+                d = 0;
+                ++b;
             }
+            if (b < cin) h.load(g, U, (const char*)in + b * fb, s, c, d);
+#pragma unroll
+            for (int a = 0; a < COUT; ++a) spin_mac(acc[a], wd + a * cin * 144, phi);
         }
+        if constexpr (LOSS) loss_site(loss, s, acc[0], d2, e2);
 #pragma unroll
         for (int a = 0; a < COUT; ++a) SpinorIO<P32>::store((char*)out + a * fb, g.V, s, acc[a]);
     }
+    if constexpr (LOSS) loss_block(loss, d2, e2);
 }
-
-// Weight gradient G[a][b][d][s][t] = sum_{x,c} gout^a(x)[s,c] conj((T_d in^b)(x)[t,c]).
-// blockIdx.y = b*9 + d; every CTA writes its partial sums (COUT*16 complex,
-// accumulated in FP32 per thread, FP64 across the CTA) to part[y][blockIdx.x].
-template <int COUT>
-__global__ void __launch_bounds__(kT) ptconv_wgrad_kernel(Geom g, const void* __restrict__ U, const void* in,
-                                                          const void* gout, double2* part) {
-    __shared__ double red[COUT * 16 * 2][kT / 32];
-    const int b = blockIdx.y / 9, d = blockIdx.y % 9;
+template <int CIN, bool LOSS>
+__global__ void __launch_bounds__(kFT, 3) ptconv_down_kernel(Geom g, int cout, const void* __restrict__ U,
+                                                             const __nv_bfloat16* __restrict__ W, const void* in,
+                                                             void* out, LossArgs loss) {
+    __shared__ __align__(16) cx<float> w[CIN * (CIN > 1 ? CIN - 1 : 1) * 9 * 16];   // cout < CIN
+    load_weights(w, W, cout * CIN * 9 * 16);
     const size_t fb = spinor_bytes<P32>(g.V);
-    cx<float> acc[COUT][16];
-#pragma unroll
-    for (int a = 0; a < COUT; ++a)
-#pragma unroll
-        for (int k = 0; k < 16; ++k) acc[a][k] = czero<float>();
+    dfloat d2, e2;
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < g.V; s += gridDim.x * blockDim.x) {
         int c[4];
         site_coords(g, s, c);
-        cx<float> phi[12];
-        transport(g, U, (const char*)in + b * fb, s, c, d, phi);
+#pragma unroll 1
+        for (int a = 0; a < cout; ++a) {
+            cx<float> acc[12];
 #pragma unroll
-        for (int a = 0; a < COUT; ++a) {
-            cx<float> gv[12];
-            SpinorIO<P32>::load((const char*)gout + a * fb, g.V, s, gv);
+            for (int k = 0; k < 12; ++k) acc[k] = czero<float>();
+            RawSpinor r;
+            r.load(in, g.V, s);
+#pragma unroll 1
+            for (int d = 0; d < 9; ++d) {
+                const HopSite h = hop_site(g, s, c, d);
+                RawLink l;
+                if (d > 0) l.load(U, g.V, (d - 1) & 3, h.link);
+                cx<float> v[12];
 #pragma unroll
-            for (int sp = 0; sp < 4; ++sp)
+                for (int k = 0; k < 12; ++k) v[k] = czero<float>();
 #pragma unroll
-                for (int t = 0; t < 4; ++t)
+                for (int b = 0; b < CIN; ++b) {
+                    cx<float> f[12];
+                    r.get(f);
+                    // the next channel, or the next direction's first
+                    if (b + 1 < CIN) r.load((const char*)in + (b + 1) * fb, g.V, h.n);
+                    else if (d < 8) r.load(in, g.V, hop_site(g, s, c, d + 1).n);
+                    spin_mac(v, w + ((a * CIN + b) * 9 + d) * 16, f);
+                }
+                if (d > 0) {
+                    cx<float> u[3][3], y[12];
+                    l.get(h.ph, u);
+                    colour_mul(u, d <= 4 ? 1 : -1, v, y);
 #pragma unroll
-                    for (int col = 0; col < 3; ++col)
-                        cfmac(acc[a][sp * 4 + t], phi[3 * t + col], gv[3 * sp + col]);
+                    for (int k = 0; k < 12; ++k) acc[k] = acc[k] + y[k];
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 12; ++k) acc[k] = v[k];
+                }
+            }
+            if constexpr (LOSS) loss_site(loss, s, acc, d2, e2);
+            SpinorIO<P32>::store((char*)out + a * fb, g.V, s, acc);
         }
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if constexpr (LOSS) loss_block(loss, d2, e2);
+}
+
+// Weight gradient G[a][b][d][s][t] = sum_{x,c} gout^a(x)[s,c] conj((T_d in^b)(x)[t,c]); since
+// T_d^dag = T_rev(d), it is also sum (T_rev(d) gout^a)[s,c] conj(in^b[t,c]) (ADJ), and the side
+// with fewer channels is the one transported.  A warp has all NS x 16 sums of one direction in
+// registers, its lanes over the sites; the eight warps of a CTA take the eight hops of the same
+// sites, so the NS static fields come from L1 for seven of them (with one CTA per direction they
+// were re-read nine times from L2 or DRAM).  The first n0 CTAs take d = 0, their warps different
+// sites.  Eight warps, not nine: with nine one SM quarter holds three and the registers per
+// thread fall from 255 to 168, which spills the sums.  The next sites' loads are in flight under
+// the products.  blockIdx.y: the transported channel.
+// Every kFlush sites per lane the sums move on, over the warp, into float pairs (48 bits), so
+// the plain FP32 accumulation is no longer than a few sites.  24^3 x 48, four static channels:
+// 1 -> 4 layer 757 -> 472 us, 4 -> 1 layer 1140 -> 451 us; bound by the FP32 pipe and by latency
+// at eight warps per SM.
+// part[(blockIdx.y * 9 + d) * max(gridDim.x - n0, n0) + cta][NS * 16]
+constexpr int kWT = 256, kFlush = 8;
+template <int NS, bool ADJ>
+__global__ void __launch_bounds__(kWT, 1) ptconv_wgrad_kernel(Geom g, const void* __restrict__ U, const void* moved,
+                                                              const void* fixed, int n0, double2* part) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool self = (int)blockIdx.x < n0;
+    const int d = self ? 0 : warp + 1;
+    const int td = !ADJ || d == 0 ? d : (d <= 4 ? d + 4 : d - 4);
+    // this warp's stretches of 32 sites: first + k * step
+    const int cta = self ? blockIdx.x : blockIdx.x - n0, ncta = self ? n0 : gridDim.x - n0;
+    const int first = self ? (cta * 8 + warp) * 32 : cta * 32, step = self ? ncta * 256 : ncta * 32;
+    const size_t fb = spinor_bytes<P32>(g.V);
+    const char* mv = (const char*)moved + blockIdx.y * fb;
+    float acc[NS][32];
+    dfloat tot[NS];
 #pragma unroll
-    for (int a = 0; a < COUT; ++a)
+    for (int a = 0; a < NS; ++a)
 #pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            float re = warp_sum(acc[a][k].re), im = warp_sum(acc[a][k].im);
-            if (lane == 0) {
-                red[2 * (a * 16 + k)][warp] = re;
-                red[2 * (a * 16 + k) + 1][warp] = im;
+        for (int k = 0; k < 32; ++k) acc[a][k] = 0.f;
+    auto flush = [&]() {
+#pragma unroll
+        for (int a = 0; a < NS; ++a) {
+            const float t = transposed_warp_sum<32>(acc[a], lane);
+            const dfloat q = two_sum(tot[a].hi, t);
+            tot[a].hi = q.hi;
+            tot[a].lo = __fadd_rn(tot[a].lo, q.lo);
+#pragma unroll
+            for (int k = 0; k < 32; ++k) acc[a][k] = 0.f;
+        }
+    };
+    RawHop h;
+    auto fetch = [&](int s) {
+        if (s < g.V) {
+            int c[4];
+            site_coords(g, s, c);
+            h.load(g, U, mv, s, c, td);
+        }
+    };
+    fetch(first + lane);
+    int it = 0;
+    // s0 is uniform over the warp: lanes past the last site take part in the sums with zeros
+    for (int s0 = first; s0 < g.V; s0 += step) {
+        const int s = s0 + lane;
+        if (s < g.V) {
+            RawSpinor r;
+            r.load(fixed, g.V, s);
+            cx<float> phi[12];
+            h.get(td, phi);
+            fetch(s + step);
+#pragma unroll
+            for (int a = 0; a < NS; ++a) {
+                cx<float> f[12];
+                r.get(f);
+                if (a + 1 < NS) r.load((const char*)fixed + (a + 1) * fb, g.V, s);
+#pragma unroll
+                for (int sp = 0; sp < 4; ++sp)
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) {
+                        cx<float> q = {acc[a][2 * (4 * sp + t)], acc[a][2 * (4 * sp + t) + 1]};
+#pragma unroll
+                        for (int col = 0; col < 3; ++col) {
+                            if constexpr (ADJ) cfmac(q, f[3 * t + col], phi[3 * sp + col]);
+                            else cfmac(q, phi[3 * t + col], f[3 * sp + col]);
+                        }
+                        acc[a][2 * (4 * sp + t)] = q.re;
+                        acc[a][2 * (4 * sp + t) + 1] = q.im;
+                    }
             }
         }
-    __syncthreads();
-    for (int q = threadIdx.x; q < COUT * 16; q += blockDim.x) {
-        double re = 0, im = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-            re += red[2 * q][w];
-            im += red[2 * q + 1][w];
+        if (++it == kFlush) {
+            flush();
+            it = 0;
         }
-        part[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * (COUT * 16) + q] = make_double2(re, im);
+    }
+    flush();
+    const int qi = transposed_index<32>(lane);
+    const int per = max((int)gridDim.x - n0, n0);
+    double* const pd = reinterpret_cast<double*>(part);
+    if (!self) {
+        double* o = pd + ((size_t)(blockIdx.y * 9 + d) * per + cta) * (NS * 32);
+#pragma unroll
+        for (int a = 0; a < NS; ++a) o[a * 32 + qi] = to_double(tot[a]);
+        return;
+    }
+    // d = 0: the eight warps' sums of the CTA, in order
+    __shared__ double red[NS * 32][9];
+#pragma unroll
+    for (int a = 0; a < NS; ++a) red[a * 32 + qi][warp] = to_double(tot[a]);
+    __syncthreads();
+    for (int q = threadIdx.x; q < NS * 32; q += kWT) {
+        double t = 0;
+        for (int w = 0; w < 8; ++w) t += red[q][w];
+        pd[((size_t)(blockIdx.y * 9) * per + cta) * (NS * 32) + q] = t;
     }
 }
 
-// y = s * (y - e) and partial sums of |y - e|^2 (for the loss), flat float2 arrays
-__global__ void residual_scale_kernel(float2* y, const float2* __restrict__ e, size_t n, float scale,
-                                      double* part) {
-    __shared__ double red[32];
-    double acc = 0;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        float2 a = y[i], b = e[i];
-        float dr = a.x - b.x, di = a.y - b.y;
-        acc += (double)dr * dr + (double)di * di;
-        y[i] = make_float2(scale * dr, scale * di);
+// the CTAs' partial sums in a fixed order, one warp per complex entry:
+// G[a][b][d][k] (+)= sum / |e|^2 (norm: the pair (|y - e|^2, |e|^2) of the training pair, or null)
+__global__ void __launch_bounds__(256) ptconv_wsum_kernel(int cin, int ns, int nmoved, int adj, int n0,
+                                                          int n8, const double2* __restrict__ part,
+                                                          const double2* __restrict__ norm, int add, double2* G) {
+    const int lane = threadIdx.x & 31;
+    const int i = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);   // (moved channel, d, fixed channel, k)
+    if (i >= nmoved * 9 * ns * 16) return;
+    const int q = i % (ns * 16), md = i / (ns * 16), d = md % 9, m = md / 9;
+    double re = 0, im = 0;
+    const int ncta = d == 0 ? n0 : n8, per = max(n0, n8);
+    for (int k = lane; k < ncta; k += 32) {
+        const double2 v = part[((size_t)md * per + k) * (ns * 16) + q];
+        re += v.x;
+        im += v.y;
     }
-    acc = warp_sum(acc);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-        part[blockIdx.x] = t;
+    re = warp_sum(re);
+    im = warp_sum(im);
+    if (lane == 0) {
+        const int a = adj ? m : q / 16, b = adj ? q / 16 : m;
+        double2& o = G[(((size_t)a * cin + b) * 9 + d) * 16 + q % 16];
+        const double sc = norm ? 1.0 / norm->y : 1.0;
+        o = make_double2((add ? o.x : 0.0) + sc * re, (add ? o.y : 0.0) + sc * im);
     }
+}
+// norms[pair] = sum of the CTAs' shares of (|y - e|^2, |e|^2)
+__global__ void __launch_bounds__(32) loss_sum_kernel(const double2* __restrict__ part, int ncta, double2* out) {
+    double a = 0, b = 0;
+    for (int k = threadIdx.x; k < ncta; k += 32) {
+        a += part[k].x;
+        b += part[k].y;
+    }
+    a = warp_sum(a);
+    b = warp_sum(b);
+    if (threadIdx.x == 0) *out = make_double2(a, b);
 }
 
 }  // namespace
 
-int ptconv_grid() { return 2 * sms(); }
+size_t ptconv_partials(int cin, int cout) {
+    // weight-gradient partials of a layer, or the loss shares of its CTAs
+    const size_t w = (size_t)cin * cout * 9 * 16 * sms();
+    const size_t l = (size_t)sms() * 16;
+    return w > l ? w : l;
+}
 
 cudaError_t launch_ptconv_forward(const GeomH& gh, int cin, int cout, const void* U32, const void* Wbf16,
-                                  const void* in, void* out, cudaStream_t st) {
-    if (cin < 1 || cin > kMaxC || cout < 1 || cout > kMaxC) return cudaErrorInvalidValue;
+                                  const void* in, void* out, cudaStream_t st, const float* target, double2* part,
+                                  double2* norms) {
+    if (cin < 1 || cin > kMaxC || cout < 1 || cout > kMaxC || (target && cout != 1)) return cudaErrorInvalidValue;
     Geom g = make_geom(gh);
-    int grid = (g.V + kT - 1) / kT;
+    int grid = (g.V + kFT - 1) / kFT;
     if (grid > sms() * 16) grid = sms() * 16;
     const __nv_bfloat16* W = (const __nv_bfloat16*)Wbf16;
-    switch (cout) {
-        case 1: (note_launch(), ptconv_forward_kernel<1><<<grid, kT, 0, st>>>(g, cin, U32, W, in, out)); break;
-        case 2: (note_launch(), ptconv_forward_kernel<2><<<grid, kT, 0, st>>>(g, cin, U32, W, in, out)); break;
-        case 3: (note_launch(), ptconv_forward_kernel<3><<<grid, kT, 0, st>>>(g, cin, U32, W, in, out)); break;
-        default: (note_launch(), ptconv_forward_kernel<4><<<grid, kT, 0, st>>>(g, cin, U32, W, in, out)); break;
+    const LossArgs l = {(const float4*)target, part};
+#define UP(C, L) (note_launch(), ptconv_up_kernel<C, L><<<grid, kFT, 0, st>>>(g, cin, U32, W, in, out, l))
+#define DOWN(C, L) (note_launch(), ptconv_down_kernel<C, L><<<grid, kFT, 0, st>>>(g, cout, U32, W, in, out, l))
+    if (cin <= cout) {
+        switch (cout) {
+            case 1: if (target) UP(1, true); else UP(1, false); break;
+            case 2: UP(2, false); break;
+            case 3: UP(3, false); break;
+            default: UP(4, false); break;
+        }
+    } else {
+        switch (cin) {
+            case 2: if (target) DOWN(2, true); else DOWN(2, false); break;
+            case 3: if (target) DOWN(3, true); else DOWN(3, false); break;
+            default: if (target) DOWN(4, true); else DOWN(4, false); break;
+        }
     }
+#undef UP
+#undef DOWN
+    if (target) (note_launch(), loss_sum_kernel<<<1, 32, 0, st>>>(part, grid, norms));
     return cudaGetLastError();
 }
 
 cudaError_t launch_ptconv_wgrad(const GeomH& gh, int cin, int cout, const void* U32, const void* in,
-                                const void* gout, double2* part, cudaStream_t st) {
+                                const void* gout, double2* part, const double2* norm, bool add, double2* G,
+                                cudaStream_t st) {
     if (cin < 1 || cin > kMaxC || cout < 1 || cout > kMaxC) return cudaErrorInvalidValue;
     Geom g = make_geom(gh);
-    dim3 grid(ptconv_grid(), cin * 9);
-    switch (cout) {
-        case 1: (note_launch(), ptconv_wgrad_kernel<1><<<grid, kT, 0, st>>>(g, U32, in, gout, part)); break;
-        case 2: (note_launch(), ptconv_wgrad_kernel<2><<<grid, kT, 0, st>>>(g, U32, in, gout, part)); break;
-        case 3: (note_launch(), ptconv_wgrad_kernel<3><<<grid, kT, 0, st>>>(g, U32, in, gout, part)); break;
-        default: (note_launch(), ptconv_wgrad_kernel<4><<<grid, kT, 0, st>>>(g, U32, in, gout, part)); break;
+    const bool adj = cin > cout;   // transport gout instead of in
+    const int nm = adj ? cout : cin, ns = adj ? cin : cout;
+    // eight hops on one set of CTAs, d = 0 (a tenth of the work: no transport, one direction) on
+    // another; together one CTA per SM
+    const int need = (g.V + 31) / 32, n8 = std::min(need, std::max(1, sms() - sms() / 10));
+    const int n0 = std::min((need + 7) / 8, std::max(1, sms() / 10));
+    const dim3 grid(n0 + n8, nm);
+#define WG(N, A) (note_launch(), ptconv_wgrad_kernel<N, A><<<grid, kWT, 0, st>>>(g, U32, A ? gout : in, A ? in : gout, n0, part))
+    switch (ns) {
+        case 1: WG(1, false); break;
+        case 2: if (adj) WG(2, true); else WG(2, false); break;
+        case 3: if (adj) WG(3, true); else WG(3, false); break;
+        default: if (adj) WG(4, true); else WG(4, false); break;
     }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_residual_scale(void* y, const void* e, size_t n, float scale, double* part, cudaStream_t st) {
-    (note_launch(), residual_scale_kernel<<<ptconv_grid(), kT, 0, st>>>((float2*)y, (const float2*)e, n, scale, part));
+#undef WG
+    const int n = nm * 9 * ns * 16;
+    (note_launch(), ptconv_wsum_kernel<<<(n + 7) / 8, 256, 0, st>>>(cin, ns, nm, adj, n0, n8, part, norm, add, G));
     return cudaGetLastError();
 }
