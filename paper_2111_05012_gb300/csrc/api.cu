@@ -2969,6 +2969,11 @@ amg_status amg_restrict(amg_hierarchy* h, int coarsening, const void* fine, void
     const GeomH& g = fine_geom(h);
     cudaStream_t st = (cudaStream_t)s;
     int cprec = prec == AMG_F64 ? 0 : 1;
+    if (prec == AMG_F32 && transfer_canon_supported(h->rp, cprec, fine)) {
+        // the caller's vectors as they are: no copy to the internal layout, no scratch
+        CK(launch_restrict_canon(h->rp, g, h->blk[0], h->p.nvec[0], rp_vecs(h), fine, coarse, nrhs, st));
+        return AMG_OK;
+    }
     DevBuf tmp;
     CK(tmp.ensure(fine_spinor_bytes(prec, g.V) * nrhs));
     CK(launch_pack_spinor(prec, g, fine, tmp.p, nrhs, st));
@@ -2984,6 +2989,10 @@ amg_status amg_prolong(amg_hierarchy* h, int coarsening, const void* coarse, voi
     const GeomH& g = fine_geom(h);
     cudaStream_t st = (cudaStream_t)s;
     int cprec = prec == AMG_F64 ? 0 : 1;
+    if (prec == AMG_F32 && transfer_canon_supported(h->rp, cprec, fine)) {
+        CK(launch_prolong_canon(h->rp, g, h->blk[0], h->p.nvec[0], rp_vecs(h), coarse, fine, nrhs, st));
+        return AMG_OK;
+    }
     DevBuf tmp;
     CK(tmp.ensure(fine_spinor_bytes(prec, g.V) * nrhs));
     CK(launch_prolong_fine(prec, h->rp, cprec, g, h->blk[0], h->p.nvec[0], rp_vecs(h), coarse, tmp.p, nrhs, st));

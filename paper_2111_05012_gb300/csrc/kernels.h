@@ -110,6 +110,12 @@ cudaError_t launch_restrict_fine(int fprec, int vprec, int cprec, const GeomH& g
                                  const void* vecs, const void* fine, void* coarse, int nrhs, cudaStream_t s);
 cudaError_t launch_prolong_fine(int fprec, int vprec, int cprec, const GeomH& g, const BlockH& bk, int nvec,
                                 const void* vecs, const void* coarse, void* fine, int nrhs, cudaStream_t s);
+// the same on the caller's canonical FP32 fine vectors (16-byte aligned), FP32 coarse vectors
+bool transfer_canon_supported(int vprec, int cprec, const void* fine);
+cudaError_t launch_restrict_canon(int vprec, const GeomH& g, const BlockH& bk, int nvec, const void* vecs,
+                                  const void* fine, void* coarse, int nrhs, cudaStream_t s);
+cudaError_t launch_prolong_canon(int vprec, const GeomH& g, const BlockH& bk, int nvec, const void* vecs,
+                                 const void* coarse, void* fine, int nrhs, cudaStream_t s);
 // block Gram-Schmidt (twice) in FP64 on nvec internal fine vectors; *err_flag set to 1 on rank deficiency
 cudaError_t launch_orthonormalise_fine(int vprec, const GeomH& g, const BlockH& bk, int nvec, void* vecs,
                                        int* err_flag, cudaStream_t s);

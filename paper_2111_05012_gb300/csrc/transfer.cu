@@ -94,78 +94,131 @@ template <> struct RawSite<P16> {   // three uint4 of halves, then the per-site 
 // vectors whose loads a thread keeps in flight together
 template <class PV> constexpr int kVecGroup = PV::id == 2 ? 4 : 2;
 
+// A fine vector as the caller holds it: 24 floats per site, one site after another (aligned to 16
+// bytes); blocks have runs of sites along x, so a warp's six loads use whole sectors.
+struct CanonF32 {
+    DEV static void load(const void* base, int, int s, cx<float> v[12]) {
+        const float4* p = (const float4*)base + (size_t)s * 6;
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+            const float4 t = __ldg(p + c);
+            v[2 * c] = {t.x, t.y};
+            v[2 * c + 1] = {t.z, t.w};
+        }
+    }
+    DEV static void store(void* base, int, int s, const cx<float> v[12]) {
+        float4* p = (float4*)base + (size_t)s * 6;
+#pragma unroll
+        for (int c = 0; c < 6; ++c) p[c] = make_float4(v[2 * c].re, v[2 * c].im, v[2 * c + 1].re, v[2 * c + 1].im);
+    }
+};
+
 // ------------------------------------------------------------ restriction
-// One CTA per block, one thread per site: the site's share of <X,s,i|psi> for a
-// group of test vectors (their loads in flight together), summed over the warp
-// by transposed shuffles and over the warps in shared memory.
-template <class PF, class PV, typename TC>
+// One CTA per block and group of NB right-hand sides, one thread per site: the site's share of
+// <X,s,i|psi_r> for a group of test vectors (their loads in flight together, the next group's
+// under the products of this one in a batch), summed over the warp by transposed shuffles and over the warps
+// in shared memory.  The test vectors are most of the traffic (96 or 52 bytes per site and vector
+// against 96 per right-hand side), so a batch reads them once per NB = 4 vectors; every
+// right-hand side goes through the same sums whatever NB is.  Bound by HBM: FP32 vectors,
+// 24^3 x 48, 24 of them, four right-hand sides 554 -> 339 us (1.78 GB, 262 us at the copy rate).
+// IO: the layout of the fine vectors (internal, or the caller's).
+template <class PV, int NB> constexpr int kGroupOf = NB == 4 ? 2 : kVecGroup<PV>;
+template <class PF, class PV, typename TC, int NB = 1, class IO = SpinorIO<PF>>
 DEV void restrict_body(const Geom& g, const Blocking& bk, int nvec, const void* __restrict__ vecs,
-                       const void* __restrict__ fine, void* coarse, int by, int gy) {
+                       const void* __restrict__ fine, size_t fstride, void* coarse, int nr, int by, int gy) {
     using T = typename PF::T;
-    constexpr int G = kVecGroup<PV>, NQ = 4 * G;   // per vector: d0.re, d0.im, d1.re, d1.im
+    constexpr int G = kGroupOf<PV, NB>, NQ = 4 * G * NB;   // per vector and right-hand side: d0.re, d0.im, d1.re, d1.im
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    cx<T>* part = reinterpret_cast<cx<T>*>(smem_raw);   // [nwarps][2*nvec]
+    cx<T>* part = reinterpret_cast<cx<T>*>(smem_raw);   // [nwarps][NB][2*nvec]
     T* partf = reinterpret_cast<T*>(smem_raw);
     const int nc = 2 * nvec;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const size_t vb = spinor_bytes<PV>(g.V);
     const int qi = transposed_index<NQ>(lane);
     const bool writer = (lane & (32 / NQ - 1)) == 0;
+    // the loads of the group of vectors from i0 on
+    auto fetch = [&](RawSite<PV> (&raw)[G], int i0, int s) {
+#pragma unroll
+        for (int u = 0; u < G; ++u)
+            if (i0 + u < nvec) raw[u].load((const char*)vecs + (size_t)(i0 + u) * vb, g.V, s);
+    };
     for (int Xi = by; Xi < bk.Vc; Xi += gy) {
         const int l = threadIdx.x;
         const bool active = l < bk.Vb;
         int c[4], s = 0;
-        cx<T> psi[12];
+        cx<T> psi[NB][12];
+        RawSite<PV> raw[G];
         if (active) {
             s = block_site(g, bk, Xi, l, c);
-            SpinorIO<PF>::load(fine, g.V, s, psi);
+            if (NB > 1) fetch(raw, 0, s);
+#pragma unroll
+            for (int r = 0; r < NB; ++r) {
+                if (r < nr) IO::load((const char*)fine + r * fstride, g.V, s, psi[r]);
+                else
+#pragma unroll
+                    for (int k = 0; k < 12; ++k) psi[r][k] = czero<T>();
+            }
         }
         for (int i0 = 0; i0 < nvec; i0 += G) {
-            RawSite<PV> raw[G];
-            if (active) {
-#pragma unroll
-                for (int u = 0; u < G; ++u)
-                    if (i0 + u < nvec) raw[u].load((const char*)vecs + (size_t)(i0 + u) * vb, g.V, s);
-            }
+            if (NB == 1 && active) fetch(raw, i0, s);
             T q[NQ];
 #pragma unroll
             for (int u = 0; u < G; ++u) {
-                cx<T> d0 = czero<T>(), d1 = czero<T>();
-                if (active && i0 + u < nvec) {
+                const RawSite<PV> v = raw[u];
+                if (NB > 1 && active && i0 + G + u < nvec)
+                    raw[u].load((const char*)vecs + (size_t)(i0 + G + u) * vb, g.V, s);
 #pragma unroll
-                    for (int k = 0; k < 6; ++k) {
-                        cfmac(d0, ccast<T>(raw[u].get(k)), psi[k]);
-                        cfmac(d1, ccast<T>(raw[u].get(6 + k)), psi[6 + k]);
+                for (int r = 0; r < NB; ++r) {
+                    cx<T> d0 = czero<T>(), d1 = czero<T>();
+                    if (active && i0 + u < nvec) {
+#pragma unroll
+                        for (int k = 0; k < 6; ++k) {
+                            cfmac(d0, ccast<T>(v.get(k)), psi[r][k]);
+                            cfmac(d1, ccast<T>(v.get(6 + k)), psi[r][6 + k]);
+                        }
                     }
+                    T* o = q + 4 * (u * NB + r);
+                    o[0] = d0.re;
+                    o[1] = d0.im;
+                    o[2] = d1.re;
+                    o[3] = d1.im;
                 }
-                q[4 * u] = d0.re;
-                q[4 * u + 1] = d0.im;
-                q[4 * u + 2] = d1.re;
-                q[4 * u + 3] = d1.im;
             }
             const T tot = transposed_warp_sum<NQ>(q, lane);
-            const int u = qi >> 2, comp = qi & 3, i = i0 + u;
-            if (writer && i < nvec) partf[2 * (warp * nc + (comp < 2 ? i : nvec + i)) + (comp & 1)] = tot;
+            const int r = (qi >> 2) % NB, comp = qi & 3, i = i0 + (qi >> 2) / NB;
+            if (writer && i < nvec)
+                partf[2 * ((warp * NB + r) * nc + (comp < 2 ? i : nvec + i)) + (comp & 1)] = tot;
         }
         __syncthreads();
-        for (int j = threadIdx.x; j < nc; j += blockDim.x) {
+        for (int j = threadIdx.x; j < nr * nc; j += blockDim.x) {
+            const int r = j / nc, q = j - r * nc;
             cx<T> t = czero<T>();
-            for (int w = 0; w < nw; ++w) t = t + part[w * nc + j];
-            CStore<TC>::st(coarse, (size_t)Xi * nc + j, ccast<TC>(t));
+            for (int w = 0; w < nw; ++w) t = t + part[(w * NB + r) * nc + q];
+            CStore<TC>::st(coarse, ((size_t)r * bk.Vc + Xi) * nc + q, ccast<TC>(t));
         }
         __syncthreads();
     }
 }
 
-// right-hand side = blockIdx.x (the fast grid index): the CTAs of one block for all
-// right-hand sides of a batch are launched together and read the same test-vector lines
-// at about the same time, so L2 serves the repeats and DRAM sees each line about once
-template <class PF, class PV, typename TC>
+// group of right-hand sides = blockIdx.x (the fast grid index): the CTAs of one block for all
+// groups of a batch are launched together and read the same test-vector lines at about the same
+// time, so L2 serves the repeats and DRAM sees each line about once
+template <class PF, class PV, typename TC, int NB, class IO>
+__global__ void __launch_bounds__(256, 1)
+    restrict_batch_kernel(Geom g, Blocking bk, int nvec, const void* __restrict__ vecs, const void* __restrict__ fine,
+                    size_t fstride, void* coarse, int nrhs, int per) {
+    const int r0 = blockIdx.x * per;
+    restrict_body<PF, PV, TC, NB, IO>(g, bk, nvec, vecs, (const char*)fine + r0 * fstride, fstride,
+                                      (char*)coarse + r0 * (size_t)bk.Vc * 2 * nvec * sizeof(cx<TC>),
+                                      min(per, nrhs - r0), blockIdx.y, gridDim.y);
+}
+// one right-hand side per CTA
+template <class PF, class PV, typename TC, class IO>
 __global__ void restrict_kernel(Geom g, Blocking bk, int nvec, const void* __restrict__ vecs,
-                                const void* __restrict__ fine, void* coarse) {
-    restrict_body<PF, PV, TC>(g, bk, nvec, vecs, (const char*)fine + blockIdx.x * spinor_bytes<PF>(g.V),
-                              (char*)coarse + blockIdx.x * (size_t)bk.Vc * 2 * nvec * sizeof(cx<TC>), blockIdx.y,
-                              gridDim.y);
+                                const void* __restrict__ fine, size_t fstride, void* coarse) {
+    restrict_body<PF, PV, TC, 1, IO>(g, bk, nvec, vecs, (const char*)fine + blockIdx.x * fstride, fstride,
+                                     (char*)coarse + blockIdx.x * (size_t)bk.Vc * 2 * nvec * sizeof(cx<TC>), 1,
+                                     blockIdx.y, gridDim.y);
 }
 // ragged batch: bc = R f32 for every problem in one launch (one CTA per block)
 template <class PV>
@@ -173,61 +226,93 @@ __global__ void restrict_ragged_kernel(const RaggedDev* __restrict__ d, const in
     int p, bx, gx;
     ragged_locate(off, np, p, bx, gx);
     const RaggedDev& q = d[p];
-    restrict_body<P32, PV, float>(q.g, q.bk, q.nvec, q.vecs, q.f32, q.bc, bx, gx);
+    restrict_body<P32, PV, float>(q.g, q.bk, q.nvec, q.vecs, q.f32, 0, q.bc, 1, bx, gx);
 }
 
 // ------------------------------------------------------------ prolongation
-// One CTA per block, one thread per site: psi'(x) = sum_{s,i} x_c(X, s, i) P_s v_i(x)
-// with the loads of a group of test vectors in flight together.
-template <class PF, class PV, typename TC>
+// One CTA per block and group of NB right-hand sides, one thread per site:
+// psi_r'(x) = sum_{s,i} x_c(X, s, i) P_s v_i(x), the loads of a group of test vectors in flight
+// under the products of the group before in a batch.  24^3 x 48, 24 FP32 vectors, four right-hand sides:
+// 485 -> 344 us.
+template <class PF, class PV, typename TC, int NB = 1, class IO = SpinorIO<PF>>
 DEV void prolong_body(const Geom& g, const Blocking& bk, int nvec, const void* __restrict__ vecs,
-                      const void* __restrict__ coarse, void* fine, int by, int gy) {
+                      const void* __restrict__ coarse, void* fine, size_t fstride, int nr, int by, int gy) {
     using T = typename PF::T;
-    constexpr int G = kVecGroup<PV>;
+    constexpr int G = kGroupOf<PV, NB>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    cx<T>* xc = reinterpret_cast<cx<T>*>(smem_raw);   // [2*nvec]
+    cx<T>* xc = reinterpret_cast<cx<T>*>(smem_raw);   // [2*nvec][NB]
     const int nc = 2 * nvec;
     const size_t vb = spinor_bytes<PV>(g.V);
+    // the loads of the group of vectors from i0 on
+    auto fetch = [&](RawSite<PV> (&raw)[G], int i0, int s) {
+#pragma unroll
+        for (int u = 0; u < G; ++u)
+            if (i0 + u < nvec) raw[u].load((const char*)vecs + (size_t)(i0 + u) * vb, g.V, s);
+    };
     for (int Xi = by; Xi < bk.Vc; Xi += gy) {
-        for (int j = threadIdx.x; j < nc; j += blockDim.x)
-            xc[j] = ccast<T>(CStore<TC>::ld(coarse, (size_t)Xi * nc + j));
-        __syncthreads();
         const int l = threadIdx.x;
-        if (l < bk.Vb) {
-            int c[4];
-            int s = block_site(g, bk, Xi, l, c);
-            cx<T> out[12];
+        const bool active = l < bk.Vb;
+        int c[4], s = 0;
+        RawSite<PV> raw[G];
+        if (active) {
+            s = block_site(g, bk, Xi, l, c);
+            if (NB > 1) fetch(raw, 0, s);
+        }
+        for (int j = threadIdx.x; j < NB * nc; j += blockDim.x) {
+            const int r = j / nc, q = j - r * nc;
+            xc[q * NB + r] = r < nr ? ccast<T>(CStore<TC>::ld(coarse, ((size_t)r * bk.Vc + Xi) * nc + q)) : czero<T>();
+        }
+        __syncthreads();
+        if (active) {
+            cx<T> out[NB][12];
 #pragma unroll
-            for (int k = 0; k < 12; ++k) out[k] = czero<T>();
+            for (int r = 0; r < NB; ++r)
+#pragma unroll
+                for (int k = 0; k < 12; ++k) out[r][k] = czero<T>();
             for (int i0 = 0; i0 < nvec; i0 += G) {
-                RawSite<PV> raw[G];
-#pragma unroll
-                for (int u = 0; u < G; ++u)
-                    if (i0 + u < nvec) raw[u].load((const char*)vecs + (size_t)(i0 + u) * vb, g.V, s);
+                if (NB == 1) fetch(raw, i0, s);
 #pragma unroll
                 for (int u = 0; u < G; ++u) {
-                    if (i0 + u >= nvec) break;
-                    const cx<T> a0 = xc[i0 + u], a1 = xc[nvec + i0 + u];
+                    const RawSite<PV> v = raw[u];
+                    if (NB > 1 && i0 + G + u < nvec) raw[u].load((const char*)vecs + (size_t)(i0 + G + u) * vb, g.V, s);
+                    if (i0 + u < nvec) {
 #pragma unroll
-                    for (int k = 0; k < 6; ++k) {
-                        cfma(out[k], a0, ccast<T>(raw[u].get(k)));
-                        cfma(out[6 + k], a1, ccast<T>(raw[u].get(6 + k)));
+                        for (int r = 0; r < NB; ++r) {
+                            const cx<T> a0 = xc[(i0 + u) * NB + r], a1 = xc[(nvec + i0 + u) * NB + r];
+#pragma unroll
+                            for (int k = 0; k < 6; ++k) {
+                                cfma(out[r][k], a0, ccast<T>(v.get(k)));
+                                cfma(out[r][6 + k], a1, ccast<T>(v.get(6 + k)));
+                            }
+                        }
                     }
                 }
             }
-            SpinorIO<PF>::store(fine, g.V, s, out);
+#pragma unroll
+            for (int r = 0; r < NB; ++r)
+                if (r < nr) IO::store((char*)fine + r * fstride, g.V, s, out[r]);
         }
         __syncthreads();
     }
 }
 
-// right-hand side = blockIdx.x, as in restrict_kernel
-template <class PF, class PV, typename TC>
+// group of right-hand sides = blockIdx.x, as in restrict_kernel
+template <class PF, class PV, typename TC, int NB, class IO>
+__global__ void __launch_bounds__(256, 1)
+    prolong_batch_kernel(Geom g, Blocking bk, int nvec, const void* __restrict__ vecs, const void* __restrict__ coarse,
+                   void* fine, size_t fstride, int nrhs, int per) {
+    const int r0 = blockIdx.x * per;
+    prolong_body<PF, PV, TC, NB, IO>(g, bk, nvec, vecs,
+                                     (const char*)coarse + r0 * (size_t)bk.Vc * 2 * nvec * sizeof(cx<TC>),
+                                     (char*)fine + r0 * fstride, fstride, min(per, nrhs - r0), blockIdx.y, gridDim.y);
+}
+// one right-hand side per CTA
+template <class PF, class PV, typename TC, class IO>
 __global__ void prolong_kernel(Geom g, Blocking bk, int nvec, const void* __restrict__ vecs,
-                               const void* __restrict__ coarse, void* fine) {
-    prolong_body<PF, PV, TC>(g, bk, nvec, vecs,
-                             (const char*)coarse + blockIdx.x * (size_t)bk.Vc * 2 * nvec * sizeof(cx<TC>),
-                             (char*)fine + blockIdx.x * spinor_bytes<PF>(g.V), blockIdx.y, gridDim.y);
+                               const void* __restrict__ coarse, void* fine, size_t fstride) {
+    prolong_body<PF, PV, TC, 1, IO>(g, bk, nvec, vecs,
+                                    (const char*)coarse + blockIdx.x * (size_t)bk.Vc * 2 * nvec * sizeof(cx<TC>),
+                                    (char*)fine + blockIdx.x * fstride, fstride, 1, blockIdx.y, gridDim.y);
 }
 // ragged batch: z = P xc for every problem in one launch (one CTA per block)
 template <class PV>
@@ -235,7 +320,7 @@ __global__ void prolong_ragged_kernel(const RaggedDev* __restrict__ d, const int
     int p, bx, gx;
     ragged_locate(off, np, p, bx, gx);
     const RaggedDev& q = d[p];
-    prolong_body<P32, PV, float>(q.g, q.bk, q.nvec, q.vecs, q.xc, q.z, bx, gx);
+    prolong_body<P32, PV, float>(q.g, q.bk, q.nvec, q.vecs, q.xc, q.z, 0, 1, bx, gx);
 }
 
 // ------------------------------------------------------------ orthonormalisation
@@ -456,26 +541,63 @@ __global__ void galerkin_kernel(Geom g, Blocking bk, int nvec, const void* __res
 
 int threads_for(const Blocking& bk) { return (bk.Vb + 31) / 32 * 32; }
 
-template <class PF, class PV, typename TC>
+// right-hand sides per CTA: the batch in groups of up to four, as even as they go (FP64 fields
+// and blocks of more than 256 sites take one: the registers of four do not fit)
+struct RhsSplit {
+    int groups, per;
+};
+RhsSplit split_rhs(int nrhs, int threads, bool many) {
+    if (!many || nrhs == 1 || threads > 256) return {nrhs, 1};
+    const int groups = (nrhs + 3) / 4;
+    return {groups, (nrhs + groups - 1) / groups};
+}
+
+template <class PF, class PV, typename TC, class IO = SpinorIO<PF>>
 cudaError_t restrict_impl(const GeomH& gh, const BlockH& bh, int nvec, const void* vecs, const void* fine,
                           void* coarse, int nrhs, cudaStream_t st) {
     Geom g = make_geom(gh);
     Blocking bk = make_blocking(gh, bh);
-    int th = threads_for(bk);
-    size_t smem = (size_t)(th / 32) * 2 * nvec * sizeof(cx<typename PF::T>);
-    (note_launch(), restrict_kernel<PF, PV, TC><<<dim3(nrhs, std::min(bk.Vc, 65535)), th, smem, st>>>(g, bk, nvec, vecs,
-                                                                                                 fine, coarse));
+    const int th = threads_for(bk);
+    const size_t fstride = spinor_bytes<PF>(g.V);   // canonical and internal FP32 fields have the same size
+    const RhsSplit sp = split_rhs(nrhs, th, PF::id != 0 && PV::id != 0);
+    const dim3 grid((nrhs + sp.per - 1) / sp.per, std::min(bk.Vc, 65535));
+    auto smem = [&](int nb) { return (size_t)(th / 32) * nb * 2 * nvec * sizeof(cx<typename PF::T>); };
+    note_launch();
+    if constexpr (PF::id != 0 && PV::id != 0) {
+        if (sp.per > 2) {
+            restrict_batch_kernel<PF, PV, TC, 4, IO><<<grid, th, smem(4), st>>>(g, bk, nvec, vecs, fine, fstride, coarse, nrhs, sp.per);
+            return cudaGetLastError();
+        }
+        if (sp.per == 2) {
+            restrict_batch_kernel<PF, PV, TC, 2, IO><<<grid, th, smem(2), st>>>(g, bk, nvec, vecs, fine, fstride, coarse, nrhs, sp.per);
+            return cudaGetLastError();
+        }
+    }
+    restrict_kernel<PF, PV, TC, IO><<<grid, th, smem(1), st>>>(g, bk, nvec, vecs, fine, fstride, coarse);
     return cudaGetLastError();
 }
-template <class PF, class PV, typename TC>
+template <class PF, class PV, typename TC, class IO = SpinorIO<PF>>
 cudaError_t prolong_impl(const GeomH& gh, const BlockH& bh, int nvec, const void* vecs, const void* coarse,
                          void* fine, int nrhs, cudaStream_t st) {
     Geom g = make_geom(gh);
     Blocking bk = make_blocking(gh, bh);
-    int th = threads_for(bk);
-    size_t smem = (size_t)2 * nvec * sizeof(cx<typename PF::T>);
-    (note_launch(), prolong_kernel<PF, PV, TC><<<dim3(nrhs, std::min(bk.Vc, 65535)), th, smem, st>>>(g, bk, nvec, vecs,
-                                                                                                coarse, fine));
+    const int th = threads_for(bk);
+    const size_t fstride = spinor_bytes<PF>(g.V);
+    const RhsSplit sp = split_rhs(nrhs, th, PF::id != 0 && PV::id != 0);
+    const dim3 grid((nrhs + sp.per - 1) / sp.per, std::min(bk.Vc, 65535));
+    auto smem = [&](int nb) { return (size_t)nb * 2 * nvec * sizeof(cx<typename PF::T>); };
+    note_launch();
+    if constexpr (PF::id != 0 && PV::id != 0) {
+        if (sp.per > 2) {
+            prolong_batch_kernel<PF, PV, TC, 4, IO><<<grid, th, smem(4), st>>>(g, bk, nvec, vecs, coarse, fine, fstride, nrhs, sp.per);
+            return cudaGetLastError();
+        }
+        if (sp.per == 2) {
+            prolong_batch_kernel<PF, PV, TC, 2, IO><<<grid, th, smem(2), st>>>(g, bk, nvec, vecs, coarse, fine, fstride, nrhs, sp.per);
+            return cudaGetLastError();
+        }
+    }
+    prolong_kernel<PF, PV, TC, IO><<<grid, th, smem(1), st>>>(g, bk, nvec, vecs, coarse, fine, fstride);
     return cudaGetLastError();
 }
 
@@ -511,6 +633,19 @@ cudaError_t launch_prolong_fine(int fprec, int vprec, int cprec, const GeomH& g,
     }
     if (cprec == 0) { DISPATCH_F(fprec, return prolong_impl<PF, P32, double>(g, bk, nvec, vecs, coarse, fine, nrhs, st)); }
     DISPATCH_F(fprec, return prolong_impl<PF, P32, float>(g, bk, nvec, vecs, coarse, fine, nrhs, st));
+}
+bool transfer_canon_supported(int vprec, int cprec, const void* fine) {
+    return vprec != 0 && cprec == 1 && ((uintptr_t)fine & 15) == 0;
+}
+cudaError_t launch_restrict_canon(int vprec, const GeomH& g, const BlockH& bk, int nvec, const void* vecs,
+                                  const void* fine, void* coarse, int nrhs, cudaStream_t st) {
+    if (vprec == 2) return restrict_impl<P32, P16, float, CanonF32>(g, bk, nvec, vecs, fine, coarse, nrhs, st);
+    return restrict_impl<P32, P32, float, CanonF32>(g, bk, nvec, vecs, fine, coarse, nrhs, st);
+}
+cudaError_t launch_prolong_canon(int vprec, const GeomH& g, const BlockH& bk, int nvec, const void* vecs,
+                                 const void* coarse, void* fine, int nrhs, cudaStream_t st) {
+    if (vprec == 2) return prolong_impl<P32, P16, float, CanonF32>(g, bk, nvec, vecs, coarse, fine, nrhs, st);
+    return prolong_impl<P32, P32, float, CanonF32>(g, bk, nvec, vecs, coarse, fine, nrhs, st);
 }
 cudaError_t launch_orthonormalise_fine(int vprec, const GeomH& gh, const BlockH& bh, int nvec, void* vecs,
                                        int* err, cudaStream_t st) {
