@@ -18,9 +18,17 @@
 // 8 x 8 core-matrix operand layout (K-major, no swizzle), one copy per site;
 // G as nine copies (one per direction d) of the neighbours' vectors, packed
 // once per call into the same layout with the k-groups outermost, so that
-// the nine pieces concatenate along K.  Copies of the next site overlap the
-// MMAs and the epilogue of the current one (two stages).  One thread issues
-// the 9Nc/16 MMAs (M 128, N 2P, K 16) and commits them to an mbarrier.
+// the nine pieces concatenate along K.  Six warps: one issues the copies into
+// a ring of stages (whole sites, two stages up to Nc = 48; thirds of a site,
+// three directions each, beyond, where two sites do not fit), one issues the
+// MMAs (M 128, N 2P, K 16), four run the epilogue from two accumulators in
+// tensor memory.  The neighbours' indices (four integer divisions) are found
+// before the wait for the stage, off the path from the MMAs' end to the next
+// copies.  Bound by HBM (the operator rows are read once).  8192 sites x Nc 48,
+// 16 right-hand sides: 211 -> 122 us (780 MB, 115 us at the copy rate).  Large copies stream better
+// than small ones: with a site in thirds 264 us (one warp issuing copies and
+// MMAs), the operator rows of a site in twelve copies 192 us against 174 us in
+// one.
 //
 // All waits are bounded: on a timeout the kernel records an error, waits
 // (bounded) for its own bulk copies, releases its tensor memory and returns.
@@ -29,7 +37,7 @@
 
 namespace {
 
-constexpr int kTcThreads = 128;
+constexpr int kTcThreads = 192;   // four epilogue warps, one for the MMAs, one for the copies
 constexpr long long kTcSpin = 20000000;
 
 DEV uint32_t su32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -60,6 +68,18 @@ DEV bool mb_try(uint64_t* bar, unsigned parity) {
 DEV bool mb_wait(uint64_t* bar, unsigned parity) {
     for (long long i = 0; i < kTcSpin; ++i)
         if (mb_try(bar, parity)) return true;
+    return false;
+}
+
+DEV void mb_arrive(uint64_t* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(bar)) : "memory");
+}
+// as mb_wait, giving up early once another role of the CTA has failed
+DEV bool mb_wait_or(uint64_t* bar, unsigned parity, const volatile int* fail) {
+    for (long long i = 0; i < kTcSpin; ++i) {
+        if (mb_try(bar, parity)) return true;
+        if ((i & 255) == 255 && *fail) return false;
+    }
     return false;
 }
 
@@ -121,7 +141,7 @@ HD size_t core_off(int row, int k, int kg) { return ((size_t)(row >> 3) * kg + (
 struct TcArgs {
     int L[4];
     int V, nc, nrhs, P;   // P: right-hand sides padded to 8 or 16
-    const __nv_bfloat16* img;   // [V][2nc rows][9nc] in core-matrix order
+    const __nv_bfloat16* img;   // [V][chunks][2nc rows][9nc / chunks] in core-matrix order
     const __nv_bfloat16* xp;    // [V][nc/8][2P/8][8][8]: packed neighbour vectors
     float2* y;                  // [nrhs][V][nc]
     const float2* b;            // residual form y = b - D x when non-null
@@ -143,18 +163,54 @@ DEV int tc_nbr(const TcArgs& a, int X, int d) {
     return c[0] + a.L[0] * (c[1] + a.L[1] * (c[2] + a.L[2] * c[3]));
 }
 
-// Shared-memory plan of one CTA (byte offsets).  An operator descriptor spans
-// 16 row groups (M = 128) but only the first 2Nc/8 hold operator rows: the
-// rest of the span may overlap the next buffer.
+// Shared-memory plan of one CTA: the ring of nst stages (operator chunk, then the packed vectors
+// of its directions), the mbarriers behind it.  An operator descriptor spans 16 row groups
+// (M = 128) but only the first 2Nc/8 hold operator rows: the rest of the span may overlap what
+// follows.
+constexpr int kMaxStages = 8;
+HD int tc_chunks(int nc) { return nc <= 48 ? 1 : 3; }   // pieces of a site, along K
 struct TcPlan {
-    int a0, a1;   // operator buffers (a1 == a0: one buffer)
-    int b0, b1;   // packed-vector buffers
-    int bar;      // mbarriers
+    int nst, stage;   // stages, bytes of one
+    int a_chunk;      // operator bytes of a stage
+    int bar;          // mbarriers (byte offset)
     int bytes;
 };
 
-// x [nrhs][V][nc] FP32 complex -> xp [V][nc/8][2P/8][8][8] bfloat16, row n = r (Re) / P + r (Im)
-__global__ void tc_pack_kernel(int V, int nc, int nrhs, int P, const float2* __restrict__ x, __nv_bfloat16* xp) {
+// x [nrhs][V][nc] FP32 complex -> xp [V][nc/8][2P/8][8][8] bfloat16, row n = r (Re) / P + r (Im).
+// One thread per eight consecutive entries of a site and right-hand side (64 bytes read, a
+// 16-byte row of each half written), right-hand side fastest: a warp writes whole 128-byte core
+// matrices (8192 x 48, 16 right-hand sides: 17 us, 33 us with 2-byte stores).
+__global__ void __launch_bounds__(256) tc_pack_kernel(int V, int nc, int nrhs, int P, const float2* __restrict__ x,
+                                                      __nv_bfloat16* xp) {
+    const int NG = 2 * P / 8, kg = nc / 8;
+    const size_t per = (size_t)nc * 2 * P;
+    const size_t n = (size_t)V * kg * P;
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        const int r = (int)(i % P);
+        const size_t t = i / P;
+        const int k8 = (int)(t % kg);
+        const size_t Y = t / kg;
+        __nv_bfloat162 re[4], im[4];
+        if (r < nrhs) {
+            const float4* src = reinterpret_cast<const float4*>(x + ((size_t)r * V + Y) * nc + 8 * k8);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float4 v = __ldg(src + q);
+                re[q] = __floats2bfloat162_rn(v.x, v.z);
+                im[q] = __floats2bfloat162_rn(v.y, v.w);
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) re[q] = im[q] = __floats2bfloat162_rn(0.f, 0.f);
+        }
+        const int rr = r, ri = P + r;
+        uint4* o = reinterpret_cast<uint4*>(xp + Y * per);
+        o[(size_t)(k8 * NG + (rr >> 3)) * 8 + (rr & 7)] = *reinterpret_cast<const uint4*>(re);
+        o[(size_t)(k8 * NG + (ri >> 3)) * 8 + (ri & 7)] = *reinterpret_cast<const uint4*>(im);
+    }
+}
+// the same for vectors that do not start on a 16-byte boundary
+__global__ void tc_pack_any_kernel(int V, int nc, int nrhs, int P, const float2* __restrict__ x, __nv_bfloat16* xp) {
     const int NG = 2 * P / 8;
     const size_t per = (size_t)nc * 2 * P;
     const size_t n = (size_t)V * nc * P;
@@ -174,90 +230,121 @@ template <int NP>   // NP = 2P accumulator columns (16 or 32)
 __global__ void __launch_bounds__(kTcThreads, 1) coarse_tc_kernel(TcArgs a, TcPlan pl) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     constexpr int P = NP / 2, NG = NP / 8;
-    const int nc = a.nc, K = 9 * nc, kg = K / 8;
-    const unsigned a_bytes = (unsigned)(2 * nc) * K * 2;        // operator rows of one site
+    const int nc = a.nc, K = 9 * nc;
+    const int nch = tc_chunks(nc), ndir = 9 / nch, Kc = K / nch, kgc = Kc / 8;   // one chunk
     const unsigned x_site = (unsigned)nc * NP * 2;              // packed vectors of one site
-    unsigned char* Ab[2] = {smem_raw + pl.a0, smem_raw + pl.a1};
-    unsigned char* Bb[2] = {smem_raw + pl.b0, smem_raw + pl.b1};
-    const bool dblA = pl.a1 != pl.a0;
-    uint64_t* barA = reinterpret_cast<uint64_t*>(smem_raw + pl.bar);   // [2]
-    uint64_t* barB = barA + 2;                                           // [2]
-    uint64_t* barM = barA + 4;
-    uint32_t* slot = reinterpret_cast<uint32_t*>(barA + 5);
-    int* fail = reinterpret_cast<int*>(slot + 1);
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw + pl.bar);   // [nst] copies of a stage
+    uint64_t* empty = full + kMaxStages;                                 // [nst] MMAs that read it
+    uint64_t* barM = empty + kMaxStages;                                 // [2] MMAs into accumulator 0 / 1
+    uint64_t* barE = barM + 2;                                           // [2] accumulator read by the epilogue
+    uint32_t* slot = reinterpret_cast<uint32_t*>(barE + 2);
+    volatile int* fail = reinterpret_cast<volatile int*>(slot + 1);   // a wait gave up: leave
+    volatile int* keep = fail + 1;                                       // MMAs may still write the accumulators
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int nq = 2 * nc / 32;   // quarters of the accumulator holding operator rows
+    const int nq = 2 * nc / 32;   // quarters of the accumulator holding operator rows, one epilogue warp each
 
     if (tid == 0) {
-        for (int i = 0; i < 5; ++i) mb_init(&barA[i], 1);
+        for (int i = 0; i < 2 * kMaxStages + 2; ++i) mb_init(&full[i], 1);
+        for (int i = 0; i < 2; ++i) mb_init(&barE[i], nq);
         mb_fence_init();
-        *fail = 0;
+        *fail = *keep = 0;
     }
     if (warp == 0) {
-        tm_alloc(slot, 32);
+        tm_alloc(slot, 64);
         tm_relinquish();
     }
     tc_before();
     __syncthreads();
     tc_after();
     const uint32_t tmem = *slot;
-    const uint32_t idesc = idesc_bf16(128, NP);
-    const uint32_t a_lbo = 128, a_sbo = (uint32_t)kg * 128;   // A: [m group][k group][8][8]
-    const uint32_t b_lbo = NG * 128, b_sbo = 128;             // G: [k group][n group][8][8]
-    unsigned phA[2] = {0, 0}, phB[2] = {0, 0}, phM = 0;
-    bool pendA[2] = {false, false}, pendB[2] = {false, false};   // thread 0 only
-    auto issueA = [&](int X, int s) {
-        mb_expect_tx(&barA[s], a_bytes);
-        bulk_load(Ab[s], a.img + (size_t)X * (2 * nc) * K, a_bytes, &barA[s]);
-        pendA[s] = true;
+    // a bounded wait by a whole warp, the same answer in every lane
+    auto wait = [&](uint64_t* bar, unsigned parity) {
+        return __all_sync(0xffffffffu, mb_wait_or(bar, parity, fail)) != 0;
     };
-    auto issueB = [&](int X, int s) {
-        mb_expect_tx(&barB[s], 9 * x_site);
-        for (int d = 0; d < 9; ++d)
-            bulk_load(Bb[s] + d * x_site, a.xp + (size_t)tc_nbr(a, X, d) * (x_site / 2), x_site, &barB[s]);
-        pendB[s] = true;
-    };
-    if (tid == 0 && (int)blockIdx.x < a.V) {
-        issueA(blockIdx.x, 0);
-        issueB(blockIdx.x, 0);
-    }
-    int it = 0;
-    for (int X = blockIdx.x; X < a.V; X += gridDim.x, ++it) {
-        const int sB = it & 1, sA = dblA ? (it & 1) : 0;
-        const int Xn = X + gridDim.x;
-        if (tid == 0) {
-            // the other stage's buffers were last read by the previous site's MMAs, which completed
-            if (Xn < a.V) {
-                issueB(Xn, sB ^ 1);
-                if (dblA) issueA(Xn, sA ^ 1);
-            }
-            if (mb_wait(&barA[sA], phA[sA]) && mb_wait(&barB[sB], phB[sB])) {
-                pendA[sA] = pendB[sB] = false;
-                phA[sA] ^= 1;
-                phB[sB] ^= 1;
-                tc_after();
-                const uint32_t a0 = su32(Ab[sA]), b0 = su32(Bb[sB]);
-                for (int q = 0; q < K / 16; ++q)
-                    mma_bf16(tmem, smem_desc(a0 + q * 256, a_lbo, a_sbo), smem_desc(b0 + q * 2 * NG * 128, b_lbo, b_sbo),
-                             idesc, q > 0 ? 1u : 0u);
-                mma_commit(barM);
-            } else {
+    const int step = gridDim.x, nst = pl.nst;
+    const int nchunk = (a.V - (int)blockIdx.x + step - 1) / step * nch;
+    if (warp == 5) {   // copies: chunk n is piece n % nch of site blockIdx.x + (n / nch) * step
+        int n = 0, st = 0, ch = 0, X = blockIdx.x;
+        unsigned phase = 0;   // of the stage's current use
+        for (; n < nchunk; ++n) {
+            // lane 1 + k fetches direction ndir * ch + k
+            const int nb = lane >= 1 && lane <= ndir ? tc_nbr(a, X, ndir * ch + lane - 1) : 0;
+            unsigned char* dst = smem_raw + (size_t)st * pl.stage;
+            if (n >= nst && !wait(&empty[st], phase ^ 1)) {
                 *fail = 1;
+                break;
+            }
+            if (lane == 0) {
+                mb_expect_tx(&full[st], pl.a_chunk + ndir * x_site);
+                bulk_load(dst, (const char*)a.img + ((size_t)X * nch + ch) * pl.a_chunk, pl.a_chunk, &full[st]);
+            }
+            __syncwarp();
+            if (lane >= 1 && lane <= ndir)
+                bulk_load(dst + pl.a_chunk + (lane - 1) * x_site, a.xp + (size_t)nb * (x_site / 2), x_site, &full[st]);
+            if (++st == nst) {
+                st = 0;
+                phase ^= 1;
+            }
+            if (++ch == nch) {
+                ch = 0;
+                X += step;
             }
         }
-        __syncthreads();
-        if (*fail) break;
-        if (!mb_wait(barM, phM)) atomicExch(fail, 2);
-        phM ^= 1;
-        __syncthreads();
-        if (*fail) break;
-        tc_after();
-        if (!dblA && tid == 0 && Xn < a.V) issueA(Xn, 0);   // the single operator buffer is free again
-        if (warp < nq) {
+        // our own bulk copies end before the shared memory goes away: each stage's last one
+        for (int k = max(0, n - nst); k < n; ++k) mb_wait(&full[k % nst], (k / nst) & 1);
+    } else if (warp == 4) {   // MMAs
+        const uint32_t idesc = idesc_bf16(128, NP);
+        const uint32_t a_lbo = 128, a_sbo = (uint32_t)kgc * 128;   // A: [m group][k group][8][8]
+        const uint32_t b_lbo = NG * 128, b_sbo = 128;              // G: [k group][n group][8][8]
+        int n = 0, st = 0, ch = 0, it = 0;
+        unsigned phase = 0;
+        for (; n < nchunk; ++n) {
+            const int acc = it & 1;
+            // the accumulator's previous site (two ago) has been read, the operands are here
+            bool ok = ch != 0 || it < 2 || wait(&barE[acc], ((it >> 1) - 1) & 1);
+            ok = ok && wait(&full[st], phase);
+            if (!ok) {
+                *fail = 1;
+                break;
+            }
+            tc_after();
+            if (lane == 0) {
+                const uint32_t a0 = su32(smem_raw + (size_t)st * pl.stage), b0 = a0 + pl.a_chunk;
+                for (int q = 0; q < Kc / 16; ++q)
+                    mma_bf16(tmem + 32 * acc, smem_desc(a0 + q * 256, a_lbo, a_sbo),
+                             smem_desc(b0 + q * 2 * NG * 128, b_lbo, b_sbo), idesc, ch > 0 || q > 0 ? 1u : 0u);
+                mma_commit(&empty[st]);
+                if (ch == nch - 1) mma_commit(&barM[acc]);
+            }
+            __syncwarp();
+            if (++st == nst) {
+                st = 0;
+                phase ^= 1;
+            }
+            if (++ch == nch) {
+                ch = 0;
+                ++it;
+            }
+        }
+        // the MMAs in flight end before the operands and accumulators go away (they complete in
+        // order); if that wait gives up, the accumulators are not released
+        if (n > 0 && !mb_wait(&empty[(n - 1) % nst], ((n - 1) / nst) & 1)) *keep = *fail = 1;
+    } else if (warp < nq) {
+        int it = 0;
+        for (int X = blockIdx.x; X < a.V; X += gridDim.x, ++it) {
+            const int sB = it & 1;
+            if (!wait(&barM[sB], (it >> 1) & 1)) {
+                *fail = 1;
+                break;
+            }
+            tc_after();
             uint32_t v[NP];
-            const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16);
+            const uint32_t taddr = tmem + 32 * sB + ((uint32_t)(warp * 32) << 16);
             if constexpr (NP == 32) tm_ld32(taddr, v);
             else tm_ld16(taddr, v);
+            tc_before();
+            __syncwarp();
+            if (lane == 0) mb_arrive(&barE[sB]);
             const int aa = warp * 16 + (lane & 15);
             const bool im = lane >= 16;
 #pragma unroll
@@ -273,41 +360,28 @@ __global__ void __launch_bounds__(kTcThreads, 1) coarse_tc_kernel(TcArgs a, TcPl
                 }
             }
         }
-        tc_before();
-        __syncthreads();
-        tc_after();
-    }
-    if (*fail && tid == 0) {
-        // drain our own bulk copies before the shared memory goes away
-        for (int s2 = 0; s2 < 2; ++s2) {
-            if (pendA[s2]) mb_wait(&barA[s2], phA[s2]);
-            if (pendB[s2]) mb_wait(&barB[s2], phB[s2]);
-        }
-        // a timed-out wait for the MMAs (fail 2) left them possibly still writing the
-        // accumulator: wait for their commit once more (phM was flipped after the failed
-        // wait); if that also gives up, the accumulator is not released (fail 3)
-        if (*fail == 2 && !mb_wait(barM, phM ^ 1)) *fail = 3;
-        atomicExch(a.err, 1);
     }
     tc_before();
     __syncthreads();
     tc_after();
-    if (warp == 0 && *fail != 3) tm_dealloc(tmem, 32);
+    if (tid == 0 && *fail) atomicExch(a.err, 1);
+    if (warp == 0 && !*keep) tm_dealloc(tmem, 64);
 }
 
 // operator image: row m = 32 w + l holds Re (l < 16) or Im (l >= 16) of
-// B[X][16 w + l % 16][d][col], column k = d * nc + col
+// B[X][16 w + l % 16][d][col], column k = d * nc + col, in tc_chunks pieces
 __global__ void tc_image_kernel(int V, int nc, const float2* __restrict__ B, __nv_bfloat16* img) {
-    const int K = 9 * nc, kg = K / 8;
+    const int K = 9 * nc, Kc = K / tc_chunks(nc), kgc = Kc / 8;
     const size_t per = (size_t)2 * nc * K;
     const size_t n = (size_t)V * per;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const size_t X = i / per;
         const int e = (int)(i - X * per);
-        const int m = e / K, k = e - m * K;
+        const int m = e / K, k = e - m * K, ch = k / Kc;
         const int row = (m >> 5) * 16 + (m & 15);
         const float2 v = B[((size_t)X * nc + row) * K + k];   // [X][row][d][col] = [X][row][k]
-        img[X * per + core_off(m, k, kg)] = __float2bfloat16((m & 16) ? v.y : v.x);
+        img[X * per + (size_t)ch * (2 * nc) * Kc + core_off(m, k - ch * Kc, kgc)] =
+            __float2bfloat16((m & 16) ? v.y : v.x);
     }
 }
 
@@ -349,26 +423,27 @@ cudaError_t launch_coarse_apply_tc(const GeomH& g, int nc, const void* img, cons
     a.y = (float2*)y;
     a.b = (const float2*)b;
     a.err = err;
-    const int K = 9 * nc, kg = K / 8, NP = 2 * a.P;
-    const int a_data = 2 * nc * K * 2, a_span = 16 * kg * 128, b_bytes = K * NP * 2;
-    const int kMax = 227 * 1024;
-    auto plan = [&](bool dbl) {
-        TcPlan p;
-        p.a0 = 0;
-        p.a1 = dbl ? a_data : 0;
-        p.b0 = p.a1 + a_data;
-        p.b1 = p.b0 + b_bytes;
-        p.bar = p.b1 + b_bytes;
-        const int end = p.bar + 5 * 8 + 8;
-        const int span = p.a1 + a_span;   // reach of the last operator descriptor
-        p.bytes = ((end > span ? end : span) + 127) / 128 * 128;
-        return p;
+    const int NP = 2 * a.P, Kc = 9 * nc / tc_chunks(nc);
+    const int kMax = 227 * 1024, bars = (2 * kMaxStages + 4) * 8 + 12;
+    TcPlan pl;
+    pl.a_chunk = 2 * nc * Kc * 2;
+    pl.stage = pl.a_chunk + Kc * NP * 2;   // multiples of 128 bytes for nc % 16 == 0
+    const int span = 16 * (Kc / 8) * 128;    // reach of an operator descriptor
+    auto need = [&](int nst) {
+        const int end = nst * pl.stage + bars, reach = (nst - 1) * pl.stage + span;
+        return ((end > reach ? end : reach) + 127) / 128 * 128;
     };
-    TcPlan pl = plan(true);
-    if (pl.bytes > kMax) pl = plan(false);
+    pl.nst = kMaxStages;
+    while (pl.nst > 2 && need(pl.nst) > kMax) --pl.nst;
+    pl.bar = pl.nst * pl.stage;
+    pl.bytes = need(pl.nst);
     if (pl.bytes > kMax) return cudaErrorInvalidValue;
-    (note_launch(), tc_pack_kernel<<<tc_sms() * 8, 256, 0, st>>>(g.V, nc, nrhs, a.P, (const float2*)x,
-                                                                 (__nv_bfloat16*)xpack));
+    if (((uintptr_t)x & 15) == 0)
+        (note_launch(), tc_pack_kernel<<<tc_sms() * 8, 256, 0, st>>>(g.V, nc, nrhs, a.P, (const float2*)x,
+                                                                     (__nv_bfloat16*)xpack));
+    else
+        (note_launch(), tc_pack_any_kernel<<<tc_sms() * 8, 256, 0, st>>>(g.V, nc, nrhs, a.P, (const float2*)x,
+                                                                         (__nv_bfloat16*)xpack));
     const void* fn = NP == 32 ? (const void*)coarse_tc_kernel<32> : (const void*)coarse_tc_kernel<16>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, pl.bytes);
     if (e != cudaSuccess) return e;
