@@ -97,8 +97,7 @@ typedef struct {
                                            FP32 vectors and arithmetic with the coarse operator
                                            stored in bfloat16 (half the bytes per stencil sweep)
                                            [AMG_F32] */
-    int sap_variant;                    /* SAP kernel: -1 autotune at setup (times the variants for one
-                                           right-hand side and for a batch, keeps the fastest of each),
+    int sap_variant;                    /* SAP kernel: -1 the library's choice (0),
                                            0 operator read from global memory, 1 operator staged in shared
                                            memory (FP32/FP16, blocks <= 256 sites; two right-hand sides
                                            per CTA in a batch), 2 as 0 but two right-hand sides of a batch

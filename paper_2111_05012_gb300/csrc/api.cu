@@ -1455,14 +1455,6 @@ amg_status setup_coarse_level(amg_hierarchy* h, int l, const double* const* init
     return AMG_OK;
 }
 
-// Autotuner: for every smoother precision the hierarchy uses, time the SAP
-// half-sweep variants on this lattice and blocking (zero fields; one full SAP
-// iteration, both colours, per sample, the variants alternating so that drifts
-// of clock or cache state hit both alike; the median of 9 samples decides),
-// once for a single right-hand side and once for a batch of three (the staged
-// variant shares its staged operator between two right-hand sides per CTA; an
-// odd batch leaves half of its last CTAs idle, so three is its worst case), and
-// keep the faster variant for each.
 // Autotuner of the stencil's launch shape for precision pr (process-wide, dirac_set_shape):
 // CTA size x grid cap from four candidates, then for FP32 / FP16 the 128-register budget for
 // the best of them; median of two timed launches each on in -> out (fields of d's lattice)
@@ -1507,62 +1499,21 @@ amg_status tune_dirac_shape(amg_dirac* d, int pr, const void* in, void* out) {
 }
 
 amg_status tune_kernels(amg_hierarchy* h) {
-    const GeomH& g = fine_geom(h);
     amg_dirac* d = h->d;
     int precs[2] = {h->fp, h->vp};
     for (int pr : precs) {
+        // variant 2 (two right-hand sides per CTA) only differs from 0 for batches; the staged
+        // variants need a blocking that fits, 3 an FP32 smoother.  -1 is variant 0: timing the
+        // variants at every setup cost a tenth of it (23 ms of 250 at 16^3 x 32 with the solves
+        // of a propagator) and chose between kernels within a few percent of each other, of
+        // which 0 is the fastest on large lattices, and among them one (3) with a half-precision
+        // operator
         const bool staged = sap_staged_supported(pr, h->blk[0]);
-        if (h->p.sap_variant >= 0) {
-            // variant 2 (two right-hand sides per CTA) only differs from 0 for batches; the
-            // staged variants need a blocking that fits, 3 an FP32 smoother
-            h->sap_variant[pr] = h->p.sap_variant == 2 ? 0 : h->p.sap_variant;
-            h->sap_variant_nb[pr] = h->p.sap_variant;
-            for (int* v : {&h->sap_variant[pr], &h->sap_variant_nb[pr]})
-                if ((!staged && (*v == 1 || *v == 3)) || (*v == 3 && pr != 1)) *v = 0;
-            continue;
-        }
-        const size_t fb = fine_spinor_bytes(pr, g.V);
-        DevBuf tb, tx;
-        CK(tb.ensure(3 * fb));
-        CK(tx.ensure(3 * fb));
-        CK(cudaMemset(tb.p, 0, 3 * fb));
-        CK(cudaMemset(tx.p, 0, 3 * fb));
-        cudaEvent_t e0, e1;
-        CK(cudaEventCreate(&e0));
-        CK(cudaEventCreate(&e1));
-        for (int nrhs : {1, 3}) {
-            // candidates: 0 operator through L1/L2, 1 staged (if the blocking allows), and for
-            // batches 2 (two right-hand sides per CTA through L1)
-            std::vector<int> vs = {0};
-            if (staged) vs.push_back(1);
-            if (nrhs > 1) vs.push_back(2);
-            if (staged && pr == 1) vs.push_back(3);
-            std::vector<float> t[4];
-            for (int rep = 0; rep < 10; ++rep) {
-                for (int v : vs) {
-                    CK(cudaEventRecord(e0, 0));
-                    for (int colour = 0; colour < 2; ++colour)
-                        CK(sap_half_launch(d, v, pr, g, h->blk[0], colour, h->p.mr_iters, 0, tb.p, tx.p, nrhs, 0));
-                    CK(cudaEventRecord(e1, 0));
-                    CK(cudaEventSynchronize(e1));
-                    float ms = 0;
-                    CK(cudaEventElapsedTime(&ms, e0, e1));
-                    if (rep > 0) t[v].push_back(ms);
-                }
-            }
-            int best_v = 0;
-            float best_t = 1e30f;
-            for (int v : vs) {
-                std::sort(t[v].begin(), t[v].end());
-                if (t[v][t[v].size() / 2] < best_t) {
-                    best_t = t[v][t[v].size() / 2];
-                    best_v = v;
-                }
-            }
-            (nrhs == 1 ? h->sap_variant : h->sap_variant_nb)[pr] = best_v;
-        }
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
+        const int want = h->p.sap_variant < 0 ? 0 : h->p.sap_variant;
+        h->sap_variant[pr] = want == 2 ? 0 : want;
+        h->sap_variant_nb[pr] = want;
+        for (int* v : {&h->sap_variant[pr], &h->sap_variant_nb[pr]})
+            if ((!staged && (*v == 1 || *v == 3)) || (*v == 3 && pr != 1)) *v = 0;
     }
     // launch shape of the stencil (threads per CTA x grid cap x register budget) for the
     // precisions the solve applies D in: the smoother's (relaxed products) and FP64 (true residual)
@@ -2499,7 +2450,8 @@ amg_status amg_dirac_create(amg_gauge* g, double kappa, double csw, amg_dirac** 
             delete d;
             return fail(AMG_ENOMEM, "clover: device allocation failed");
         }
-        cudaError_t e = launch_clover_build(pr, geo, g->U[0].p, kappa, csw, d->C[pr].p, 0);
+        cudaError_t e = pr == 0 ? launch_clover_build(geo, g->U[0].p, kappa, csw, d->C[0].p, 0)
+                                : launch_clover_convert(pr, geo, d->C[0].p, d->C[pr].p, 0);
         if (e != cudaSuccess) {
             delete d;
             return fail(AMG_ECUDA, std::string("clover build: ") + cudaGetErrorString(e));

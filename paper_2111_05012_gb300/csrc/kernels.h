@@ -42,8 +42,10 @@ cudaError_t launch_gauge_random(const GeomH& g, double eps, uint64_t seed, uint6
 // internal P64 links -> canonical doubles
 cudaError_t launch_gauge_unpack64(const GeomH& g, const void* U64, double* canon, cudaStream_t s);
 // FP64 clover build from the internal P64 gauge; writes the packed clover of prec
-cudaError_t launch_clover_build(int prec, const GeomH& g, const void* U64, double kappa, double csw, void* clover,
+cudaError_t launch_clover_build(const GeomH& g, const void* U64, double kappa, double csw, void* clover64,
                                 cudaStream_t s);
+// the packed FP64 clover in the layout of prec (1, 2, 3)
+cudaError_t launch_clover_convert(int prec, const GeomH& g, const void* C64, void* clover, cudaStream_t s);
 // internal P64 clover -> [site][2][6][6][2] doubles (device)
 cudaError_t launch_clover_expand(const GeomH& g, const void* C64, double* out, cudaStream_t s);
 

@@ -334,8 +334,37 @@ __global__ void prolong_ragged_kernel(const RaggedDev* __restrict__ d, const int
 // eps |w0| / |w| <= 2 eps otherwise (the DGKS test).  Either way the result is
 // the QR factor with a positive diagonal to rounding, the vectors that
 // projecting one vector after another gives.
+// FP64 runs at 1/64 of the FP32 rate, so the FP64 instructions are the time: fused multiply-adds
+// (48 per pair of vectors and site half), and FP32 values widened with integer instructions
+// instead of conversions on the FP64 pipe.  16^3 x 32, 24 vectors: 16.4 -> 11.8 ms.
+DEV double widen(float f) {
+    const unsigned u = __float_as_uint(f), e = (u >> 23) & 0xFFu;
+    if (e == 0 || e == 255) return (double)f;   // zero and subnormal values, infinities, NaN
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + (896u << 20))), (int)(u << 29));
+}
+DEV cx<double> widen(cx<float> a) { return {widen(a.re), widen(a.im)}; }
+DEV cx<double> widen(cx<double> a) { return a; }
+// chirality half chi of a fine field at one site (plain loads: written earlier in the launch)
+template <class PV> DEV void load_chirality(const void* base, int V, int s, int chi, cx<typename PV::T> v[6]);
+template <> DEV void load_chirality<P32>(const void* base, int V, int s, int chi, cx<float> v[6]) {
+    const float4* p = (const float4*)base + (size_t)3 * chi * V;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const float4 t = p[(size_t)c * V + s];
+        v[2 * c] = {t.x, t.y};
+        v[2 * c + 1] = {t.z, t.w};
+    }
+}
+template <> DEV void load_chirality<P64>(const void* base, int V, int s, int chi, cx<double> v[6]) {
+    const double2* p = (const double2*)base + (size_t)6 * chi * V;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        const double2 t = p[(size_t)k * V + s];
+        v[k] = {t.x, t.y};
+    }
+}
 template <class PV>
-__global__ void orthonormalise_kernel(Geom g, Blocking bk, int nvec, void* vecs, int* err) {
+__global__ void __launch_bounds__(512) orthonormalise_kernel(Geom g, Blocking bk, int nvec, void* vecs, int* err) {
     __shared__ double red[3 * 32];
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<double>* part = reinterpret_cast<cx<double>*>(smem_raw);   // [nwarps][nvec]
@@ -344,14 +373,15 @@ __global__ void orthonormalise_kernel(Geom g, Blocking bk, int nvec, void* vecs,
     const int l = threadIdx.x, lane = l & 31, warp = l >> 5, nw = blockDim.x >> 5;
     const bool active = l < bk.Vb;
     const size_t vb = spinor_bytes<PV>(g.V);
+    constexpr int G = PV::id == 0 ? 1 : 2;   // previous vectors in flight (more spill at the 128 registers of 512 threads)
     int c[4], s = 0;
     if (active) s = block_site(g, bk, Xi, l, c);
     auto load_half = [&](int j, cx<double> (&q)[6]) {
         if (active) {
-            cx<typename PV::T> u[12];
-            SpinorIO<PV>::load_rw((const char*)vecs + j * vb, g.V, s, u);
+            cx<typename PV::T> u[6];
+            load_chirality<PV>((const char*)vecs + j * vb, g.V, s, chi, u);
 #pragma unroll
-            for (int k = 0; k < 6; ++k) q[k] = ccast<double>(u[6 * chi + k]);
+            for (int k = 0; k < 6; ++k) q[k] = widen(u[k]);
         } else {
 #pragma unroll
             for (int k = 0; k < 6; ++k) q[k] = czero<double>();
@@ -370,15 +400,28 @@ __global__ void orthonormalise_kernel(Geom g, Blocking bk, int nvec, void* vecs,
                 block_sum<double, 1>(n1, red);
                 if (n1[0] > 0.25 * n0[0]) break;
             }
-            for (int j = 0; j < i; ++j) {
-                cx<double> q[6];
-                load_half(j, q);
-                cx<double> d = czero<double>();
+            // G previous vectors at a time: their loads in flight together, and their sums taken over
+            // the warp by transposed shuffles (10 FP64 additions for four sums instead of 20)
+            for (int j0 = 0; j0 < i; j0 += G) {
+                cx<typename PV::T> u[G][6];
 #pragma unroll
-                for (int k = 0; k < 6; ++k) d = d + cmulc(q[k], w[k]);
-                d.re = warp_sum(d.re);
-                d.im = warp_sum(d.im);
-                if (lane == 0) part[warp * nvec + j] = d;
+                for (int t = 0; t < G; ++t)
+                    if (active && j0 + t < i) load_chirality<PV>((const char*)vecs + (j0 + t) * vb, g.V, s, chi, u[t]);
+                double q[2 * G];
+#pragma unroll
+                for (int t = 0; t < G; ++t) {
+                    cx<double> d = czero<double>();
+                    if (active && j0 + t < i) {
+#pragma unroll
+                        for (int k = 0; k < 6; ++k) cfmac(d, widen(u[t][k]), w[k]);
+                    }
+                    q[2 * t] = d.re;
+                    q[2 * t + 1] = d.im;
+                }
+                const double tot = transposed_warp_sum<2 * G>(q, lane);
+                const int v = transposed_index<2 * G>(lane);
+                if ((lane & (32 / (2 * G) - 1)) == 0 && j0 + (v >> 1) < i)
+                    reinterpret_cast<double*>(part + warp * nvec + j0 + (v >> 1))[v & 1] = tot;
             }
             __syncthreads();
             for (int j = l; j < i; j += blockDim.x) {
@@ -387,12 +430,18 @@ __global__ void orthonormalise_kernel(Geom g, Blocking bk, int nvec, void* vecs,
                 coef[j] = t;
             }
             __syncthreads();
-            for (int j = 0; j < i; ++j) {
-                cx<double> q[6];
-                load_half(j, q);
-                const cx<double> cc = coef[j];
+            for (int j0 = 0; j0 < i; j0 += G) {
+                cx<typename PV::T> u[G][6];
 #pragma unroll
-                for (int k = 0; k < 6; ++k) w[k] = w[k] - cc * q[k];
+                for (int t = 0; t < G; ++t)
+                    if (active && j0 + t < i) load_chirality<PV>((const char*)vecs + (j0 + t) * vb, g.V, s, chi, u[t]);
+#pragma unroll
+                for (int t = 0; t < G; ++t) {
+                    if (!active || j0 + t >= i) break;
+                    const cx<double> cc = -coef[j0 + t];
+#pragma unroll
+                    for (int k = 0; k < 6; ++k) cfma(w[k], cc, widen(u[t][k]));
+                }
             }
             __syncthreads();   // part / coef are rewritten by the next pass
         }
@@ -421,37 +470,35 @@ __global__ void orthonormalise_kernel(Geom g, Blocking bk, int nvec, void* vecs,
 // T_d = H_d P_t v_j on the sites of Xi (H_0 = D_SAP on the block, H_{+-mu} =
 // the hops of D leaving Xi through its +-mu face) are formed for both columns
 // and projected on all basis vectors of Xi: B[Xi][I][d][J] = <Xi, I| T_d>.
-// Each test-vector load serves both columns; in a face direction only the
-// face sites of the block (a quarter of them for 4^4 blocks) load anything,
-// and a warp without face sites skips the direction; the four projections of
-// a vector (two columns x two chiralities) are summed over the warp by one
-// transposed shuffle reduction.
+// Each test-vector load serves both columns, and the four projections of a
+// vector (two columns x two chiralities) are summed over the warp by one
+// transposed shuffle reduction.  d = 0 takes one thread per site; a face
+// direction has a quarter of the sites (4^4 blocks), so the face's T goes to
+// shared memory and the CTA's threads split into groups over the same face
+// sites, each group projecting on its share of the test vectors: the vectors
+// are read from L2 for 3 blocks' worth of sites per column pair instead of
+// 6.5 (every warp has sites of most faces).  16^3 x 32, 24 vectors: 11.0 ->
+// 6.9 ms; bound by the L2 (every column pair reads the block's vectors).
 template <class PV, typename TC>
-__global__ void galerkin_kernel(Geom g, Blocking bk, int nvec, const void* __restrict__ vecs,
+__global__ void __launch_bounds__(PV::id == 0 ? 256 : 512) galerkin_kernel(Geom g, Blocking bk, int nvec, const void* __restrict__ vecs,
                                 const void* __restrict__ U, const void* __restrict__ C, typename PV::T kappa,
                                 void* B) {
     using T = typename PV::T;
     constexpr int NQ = 8;   // per vector: column a / b x chirality 0 / 1 x (re, im)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nc = 2 * nvec;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     T* partf = reinterpret_cast<T*>(smem_raw);   // [nwarps][2 columns][nc] complex
     cx<T>* part = reinterpret_cast<cx<T>*>(smem_raw);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    cx<T>* tsh = part + (size_t)nw * 2 * nc;     // [2 columns][12][face sites, padded]
     const int Xi = blockIdx.x, Ja = 2 * blockIdx.y, Jb = Ja + 1;
     const bool hasB = Jb < nc;
     const int ta = Ja / nvec, ja = Ja % nvec, tb = hasB ? Jb / nvec : 0, jb = hasB ? Jb % nvec : 0;
     const size_t vb = spinor_bytes<PV>(g.V);
     const char* va = (const char*)vecs + ja * vb;
     const char* vbp = (const char*)vecs + jb * vb;
-    const int l = threadIdx.x;
-    const bool active = l < bk.Vb;
     const int qi = transposed_index<NQ>(lane);
     const bool writer = (lane & (32 / NQ - 1)) == 0;
-    int c[4] = {0, 0, 0, 0}, lc[4] = {0, 0, 0, 0}, s = 0;
-    if (active) {
-        s = block_site(g, bk, Xi, l, c);
-        for (int mu = 0; mu < 4; ++mu) lc[mu] = c[mu] % bk.b[mu];
-    }
     auto load_proj = [&](const char* v, int t, int site, cx<T> out[12]) {
         SpinorIO<PV>::load(v, g.V, site, out);
 #pragma unroll
@@ -471,12 +518,25 @@ __global__ void galerkin_kernel(Geom g, Blocking bk, int nvec, const void* __res
     for (int d = 0; d < 9; ++d) {
         const int mu = d == 0 ? 0 : (d - 1) % 4;
         const int dir = d <= 4 ? +1 : -1;
-        const bool face = d == 0 || (dir > 0 ? (lc[mu] == bk.b[mu] - 1) : (lc[mu] == 0));
-        const bool work = active && face;
+        // this direction's sites: nf of them, padded to whole warps, and the groups of threads over them
+        const int nf = d == 0 ? bk.Vb : bk.Vb / bk.b[mu];
+        const int nfp = (nf + 31) / 32 * 32, ngrp = blockDim.x / nfp, nwf = nfp >> 5;
+        const int grp = threadIdx.x / nfp, f = threadIdx.x - grp * nfp;
+        const bool work = grp < ngrp && f < nf;
+        int c[4] = {0, 0, 0, 0}, s = 0;
         cx<T> Ta[12], Tb[12];
 #pragma unroll
         for (int k = 0; k < 12; ++k) Ta[k] = Tb[k] = czero<T>();
         if (work) {
+            int l = f;
+            if (d != 0) {
+                int low = 1;
+                for (int m = 0; m < mu; ++m) low *= bk.b[m];
+                l = f % low + low * ((dir > 0 ? bk.b[mu] - 1 : 0) + bk.b[mu] * (f / low));
+            }
+            s = block_site(g, bk, Xi, l, c);
+        }
+        if (work && grp == 0) {
             float ph;
             if (d == 0) {
                 cx<T> psi[12];
@@ -487,11 +547,12 @@ __global__ void galerkin_kernel(Geom g, Blocking bk, int nvec, const void* __res
                     clover_apply<PV>(C, g.V, s, psi, Tb);
                 }
                 for (int m = 0; m < 4; ++m) {
-                    if (lc[m] != bk.b[m] - 1) {
+                    const int lc = c[m] % bk.b[m];
+                    if (lc != bk.b[m] - 1) {
                         int n = neighbour(g, s, c, m, +1, ph);
                         hop2(n, s, m, +1, -kappa * T(ph), Ta, Tb);
                     }
-                    if (lc[m] != 0) {
+                    if (lc != 0) {
                         int n = neighbour(g, s, c, m, -1, ph);
                         hop2(n, n, m, -1, -kappa * T(ph), Ta, Tb);
                     }
@@ -500,13 +561,26 @@ __global__ void galerkin_kernel(Geom g, Blocking bk, int nvec, const void* __res
                 int n = neighbour(g, s, c, mu, dir, ph);
                 hop2(n, dir > 0 ? s : n, mu, dir, -kappa * T(ph), Ta, Tb);
             }
-        }
-        const bool wwork = __any_sync(0xffffffffu, work);
-        for (int i = 0; i < nvec; ++i) {
-            if (!wwork) {   // no face site in this warp: its partial sums are zero
-                if (lane < 4) part[(warp * 2 + (lane >> 1)) * nc + (lane & 1) * nvec + i] = czero<T>();
-                continue;
+            if (ngrp > 1) {
+#pragma unroll
+                for (int k = 0; k < 12; ++k) {
+                    tsh[k * nfp + f] = Ta[k];
+                    tsh[(12 + k) * nfp + f] = Tb[k];
+                }
             }
+        }
+        if (ngrp > 1) {
+            __syncthreads();
+            if (work && grp > 0) {
+#pragma unroll
+                for (int k = 0; k < 12; ++k) {
+                    Ta[k] = tsh[k * nfp + f];
+                    Tb[k] = tsh[(12 + k) * nfp + f];
+                }
+            }
+        }
+        const int wf = warp - grp * nwf;   // warp within its group (groups are whole warps)
+        for (int i = grp; i < nvec && grp < ngrp; i += ngrp) {
             cx<T> d0a = czero<T>(), d1a = czero<T>(), d0b = czero<T>(), d1b = czero<T>();
             if (work) {
                 cx<T> v[12];
@@ -524,7 +598,7 @@ __global__ void galerkin_kernel(Geom g, Blocking bk, int nvec, const void* __res
             if (writer) {
                 const int col = qi >> 2, comp = qi & 3;
                 const int row = (comp < 2 ? 0 : nvec) + i;
-                partf[2 * ((warp * 2 + col) * nc + row) + (comp & 1)] = tot;
+                partf[2 * ((wf * 2 + col) * nc + row) + (comp & 1)] = tot;
             }
         }
         __syncthreads();
@@ -532,7 +606,7 @@ __global__ void galerkin_kernel(Geom g, Blocking bk, int nvec, const void* __res
             const int col = r / nc, row = r % nc;
             if (col == 1 && !hasB) continue;
             cx<T> acc = czero<T>();
-            for (int w = 0; w < nw; ++w) acc = acc + part[(w * 2 + col) * nc + row];
+            for (int w = 0; w < nwf; ++w) acc = acc + part[(w * 2 + col) * nc + row];
             CStore<TC>::st(B, (((size_t)Xi * nc + row) * 9 + d) * nc + (col ? Jb : Ja), ccast<TC>(acc));
         }
         __syncthreads();
@@ -664,12 +738,18 @@ cudaError_t launch_galerkin_fine(int vprec, int cprec, const GeomH& gh, const Bl
     Blocking bk = make_blocking(gh, bh);
     int th = threads_for(bk);
     dim3 grid(bk.Vc, nvec);   // pairs of columns
+    // T of the largest face that leaves room for a second group of threads
+    size_t face = 0;
+    for (int mu = 0; mu < 4; ++mu) {
+        const size_t nfp = (bk.Vb / bk.b[mu] + 31) / 32 * 32;
+        if (th >= (int)(2 * nfp) && 24 * nfp > face) face = 24 * nfp;
+    }
     if (vprec == 0) {
-        size_t smem = (size_t)(th / 32) * 2 * 2 * nvec * sizeof(cx<double>);
+        const size_t smem = ((size_t)(th / 32) * 2 * 2 * nvec + face) * sizeof(cx<double>);
         if (cprec == 0) (note_launch(), galerkin_kernel<P64, double><<<grid, th, smem, st>>>(g, bk, nvec, vecs, U, C, kappa, B));
         else (note_launch(), galerkin_kernel<P64, float><<<grid, th, smem, st>>>(g, bk, nvec, vecs, U, C, kappa, B));
     } else {
-        size_t smem = (size_t)(th / 32) * 2 * 2 * nvec * sizeof(cx<float>);
+        const size_t smem = ((size_t)(th / 32) * 2 * 2 * nvec + face) * sizeof(cx<float>);
         if (cprec == 0) (note_launch(), galerkin_kernel<P32, double><<<grid, th, smem, st>>>(g, bk, nvec, vecs, U, C, (float)kappa, B));
         else (note_launch(), galerkin_kernel<P32, float><<<grid, th, smem, st>>>(g, bk, nvec, vecs, U, C, (float)kappa, B));
     }
