@@ -97,14 +97,11 @@ typedef struct {
                                            FP32 vectors and arithmetic with the coarse operator
                                            stored in bfloat16 (half the bytes per stencil sweep)
                                            [AMG_F32] */
-    int sap_variant;                    /* SAP kernel: -1 the library's choice (0),
-                                           0 operator read from global memory, 1 operator staged in shared
-                                           memory (FP32/FP16, blocks <= 256 sites; two right-hand sides
-                                           per CTA in a batch), 2 as 0 but two right-hand sides of a batch
-                                           per CTA sharing the operator in L1 (FP32/FP16, <= 256 sites),
-                                           3 FP32 smoother with the operator staged in shared memory from
-                                           its FP16 copy (<= 256 sites; residual with the FP32 operator)
-                                           [-1] */
+    int sap_variant;                    /* SAP kernel, -1..3: 3 takes the minimal-residual steps' operator
+                                           from its FP16 copy (FP32 smoother, blocks <= 256 sites;
+                                           residual with the FP32 operator); every other value the
+                                           operator in the smoother's precision (-1, 0, 1 and 2 once
+                                           chose among kernels that one has since replaced) [-1] */
     int outer_solver;                   /* 0: flexible GMRES(outer_m) [0]; 1: the paper's BiCGStab with
                                            flexible preconditioning (Sec. 3), one right-hand side at a
                                            time; 2: the paper's comparison solver MBiCGs (Sec. 5,

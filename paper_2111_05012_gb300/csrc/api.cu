@@ -247,8 +247,6 @@ struct amg_hierarchy {
     DevBuf err_flag;
     DevBuf ac_in, ac_out;   // amg_apply_coarse: vectors converted to the level's precision (kept)
     int coarse_cycles = 0;
-    int sap_variant[3] = {0, 0, 0};      // chosen SAP kernel per smoother precision, one right-hand side
-    int sap_variant_nb[3] = {0, 0, 0};   // the same for batches (the staged kernel then takes two per CTA)
     amg_nn* nn = nullptr;             // learned correction after the cycle (FP32 smoother only)
     bool nn_off = false;              // set while falling back to the plain cycle
     int* hstate = nullptr;   // pinned mirror of the coarse solver state words (16 x 4 ints)
@@ -382,21 +380,11 @@ amg_status true_residual(amg_hierarchy* h, const void* x, void* r, const void* b
     return fine_D(h, 0, x, r, b, nb, s);
 }
 
-// one SAP half sweep with kernel variant var (0-2: launch_sap_half_variant; 3: FP32 vectors
-// with the domain operator staged from its FP16 copy)
-cudaError_t sap_half_launch(amg_dirac* d, int var, int prec, const GeomH& g, const BlockH& bk, int colour, int nmr,
-                            int x_mode, const void* b, void* x, int nb, cudaStream_t s) {
-    if (var == 3 && prec == 1)
-        return launch_sap_half_staged16(g, bk, colour, nmr, x_mode, d->gauge->U[1].p, d->C[1].p, d->gauge->U[2].p,
-                                        d->C[2].p, b, x, d->kappa, nb, s);
-    return launch_sap_half_variant(var == 3 ? 1 : var, prec, g, bk, colour, nmr, x_mode, d->gauge->U[prec].p,
-                                   d->C[prec].p, b, x, d->kappa, nb, s);
-}
-
 amg_status fine_sap(amg_hierarchy* h, int prec, const void* b, void* x, bool x_zero, int nb, cudaStream_t s) {
     amg_dirac* d = h->d;
     h->timer.start(PH_SMOOTH, s);
-    const int var = nb > 1 ? h->sap_variant_nb[prec] : h->sap_variant[prec];
+    // sap_variant 3: the FP16 copy of the operator under FP32 vectors
+    const bool op16 = h->p.sap_variant == 3 && prec == 1 && sap_staged_supported(1, h->blk[0]);
     for (int i = 0; i < h->p.sap_iters; ++i) {
         const bool first = x_zero && i == 0;
         for (int colour = 0; colour < 2; ++colour) {
@@ -404,9 +392,12 @@ amg_status fine_sap(amg_hierarchy* h, int prec, const void* b, void* x, bool x_z
             if (h->p.sap_eo)
                 CK(launch_sap_half_eo(prec, fine_geom(h), h->blk[0], colour, h->p.mr_iters, x_mode,
                                       d->gauge->U[prec].p, d->C[prec].p, d->Ci[prec].p, b, x, d->kappa, nb, s));
+            else if (op16)
+                CK(launch_sap_half_staged16(fine_geom(h), h->blk[0], colour, h->p.mr_iters, x_mode, d->gauge->U[1].p,
+                                            d->C[1].p, d->gauge->U[2].p, d->C[2].p, b, x, d->kappa, nb, s));
             else
-                CK(sap_half_launch(d, var, prec, fine_geom(h), h->blk[0], colour, h->p.mr_iters, x_mode, b, x, nb,
-                                   s));
+                CK(launch_sap_half(prec, fine_geom(h), h->blk[0], colour, h->p.mr_iters, x_mode,
+                                   d->gauge->U[prec].p, d->C[prec].p, b, x, d->kappa, nb, s));
         }
     }
     if (h->p.sap_iters == 0 && x_zero) CK(cudaMemsetAsync(x, 0, fsz(h, prec) * nb, s));
@@ -1500,21 +1491,6 @@ amg_status tune_dirac_shape(amg_dirac* d, int pr, const void* in, void* out) {
 
 amg_status tune_kernels(amg_hierarchy* h) {
     amg_dirac* d = h->d;
-    int precs[2] = {h->fp, h->vp};
-    for (int pr : precs) {
-        // variant 2 (two right-hand sides per CTA) only differs from 0 for batches; the staged
-        // variants need a blocking that fits, 3 an FP32 smoother.  -1 is variant 0: timing the
-        // variants at every setup cost a tenth of it (23 ms of 250 at 16^3 x 32 with the solves
-        // of a propagator) and chose between kernels within a few percent of each other, of
-        // which 0 is the fastest on large lattices, and among them one (3) with a half-precision
-        // operator
-        const bool staged = sap_staged_supported(pr, h->blk[0]);
-        const int want = h->p.sap_variant < 0 ? 0 : h->p.sap_variant;
-        h->sap_variant[pr] = want == 2 ? 0 : want;
-        h->sap_variant_nb[pr] = want;
-        for (int* v : {&h->sap_variant[pr], &h->sap_variant_nb[pr]})
-            if ((!staged && (*v == 1 || *v == 3)) || (*v == 3 && pr != 1)) *v = 0;
-    }
     // launch shape of the stencil (threads per CTA x grid cap x register budget) for the
     // precisions the solve applies D in: the smoother's (relaxed products) and FP64 (true residual)
     for (int pr : {h->fp, 0}) TRY(tune_dirac_shape(d, pr, h->fx[pr].p, h->fb[pr].p));

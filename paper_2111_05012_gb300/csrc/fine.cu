@@ -1086,6 +1086,166 @@ __global__ void clover_invert_kernel(Geom g, const void* C64, void* out) {
     }
 }
 
+// ------------------------------------------------------------ FP32 spinors in packed pairs
+// (re, im) as one 64-bit register pair and the .f32x2 instructions: one instruction per complex
+// component pair.  The FP32 pipe does the same multiply-adds per clock either way (74 TFLOP/s
+// measured both ways), but the SAP kernel issues on 57 % of its cycles at 47 % of that rate, so
+// halving the multiply-add instructions is what can be had.  Broadcasting one half of a register
+// pair and swapping the two are free operand forms; negating a half is not (two to four integer
+// instructions), so a complex product a b = a.re (b.re, b.im) + a.im (-b.im, b.re) takes its
+// second factor's rotated form rot(b), one multiplication by (-1, 1), and every b here is used
+// with three or more a.
+struct f2 {
+    unsigned long long v;
+};
+DEV f2 pk2(float a, float b) {
+    f2 d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d.v) : "f"(a), "f"(b));
+    return d;
+}
+DEV void unpk2(f2 p, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(p.v)); }
+DEV f2 dup2(float a) { return pk2(a, a); }
+DEV f2 swap2(f2 p) {
+    float a, b;
+    unpk2(p, a, b);
+    return pk2(b, a);
+}
+DEV f2 fma2(f2 a, f2 b, f2 c) {
+    f2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return d;
+}
+DEV f2 mul2(f2 a, f2 b) {
+    f2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d.v) : "l"(a.v), "l"(b.v));
+    return d;
+}
+DEV f2 add2(f2 a, f2 b) {
+    f2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d.v) : "l"(a.v), "l"(b.v));
+    return d;
+}
+DEV f2 pm2() { return pk2(1.f, -1.f); }
+DEV f2 mp2() { return pk2(-1.f, 1.f); }
+DEV f2 rot2(f2 b) { return mul2(mp2(), swap2(b)); }    // i b
+DEV f2 nrot2(f2 b) { return mul2(pm2(), swap2(b)); }   // -i b
+
+// a spinor as six 16-byte words
+DEV void spinor_pairs(const float4 (&t)[6], f2 v[12]) {
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        v[2 * c] = pk2(t[c].x, t[c].y);
+        v[2 * c + 1] = pk2(t[c].z, t[c].w);
+    }
+}
+template <class P> DEV void load_pairs(const void* base, int V, int s, f2 v[12]) {
+    cx<float> t[12];
+    SpinorIO<P>::load(base, V, s, t);
+#pragma unroll
+    for (int k = 0; k < 12; ++k) v[k] = pk2(t[k].re, t[k].im);
+}
+DEV void tile_put(float4* p, int vbp, int l, const f2 v[12]) {
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        float4 t;
+        unpk2(v[2 * c], t.x, t.y);
+        unpk2(v[2 * c + 1], t.z, t.w);
+        p[c * vbp + l] = t;
+    }
+}
+DEV void tile_get(const float4* p, int vbp, int l, f2 v[12]) {
+    float4 t[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) t[c] = p[c * vbp + l];
+    spinor_pairs(t, v);
+}
+
+// out[0..5] = A_b in[0..5] (clover_block_apply)
+DEV void clover_pairs(const float pr[36], const f2* in, f2* out) {
+    f2 ro[6], nr[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        out[i] = mul2(dup2(pr[i]), in[i]);
+        ro[i] = rot2(in[i]);
+        nr[i] = nrot2(in[i]);
+    }
+#pragma unroll
+    for (int i = 1; i < 6; ++i)
+#pragma unroll
+        for (int j = 0; j < i; ++j) {
+            const int q = 3 + i * (i - 1) / 2 + j;
+            const f2 lr = dup2(pr[2 * q]), li = dup2(pr[2 * q + 1]);
+            out[i] = fma2(lr, in[j], out[i]);
+            out[i] = fma2(li, ro[j], out[i]);
+            out[j] = fma2(lr, in[i], out[j]);
+            out[j] = fma2(li, nr[i], out[j]);
+        }
+}
+
+// out += coeff (1 - dir gamma_mu) W psi, W = U (dir = +1) or U^dag (dir = -1) (hop_accum); mu and
+// dir are compile-time constants after unrolling
+DEV void hop_pairs(f2 out[12], const f2 psi[12], const cx<float> u[3][3], int mu, int dir, float coeff) {
+    f2 w0[3], w1[3];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        // h = upper -/+ e_mu lower, one colour
+        const f2 v0 = psi[6 + b], v1 = psi[9 + b];
+        const f2 s = dir > 0 ? pm2() : mp2(), n1 = dup2(-1.f);   // -/+ i x = s * swap(x)
+        f2 h0, h1;
+        switch (mu) {
+            case 0: h0 = fma2(s, swap2(v1), psi[b]); h1 = fma2(s, swap2(v0), psi[3 + b]); break;
+            case 1:
+                h0 = dir > 0 ? fma2(n1, v1, psi[b]) : add2(psi[b], v1);
+                h1 = dir > 0 ? add2(psi[3 + b], v0) : fma2(n1, v0, psi[3 + b]);
+                break;
+            case 2:
+                h0 = fma2(s, swap2(v0), psi[b]);
+                h1 = fma2(dir > 0 ? mp2() : pm2(), swap2(v1), psi[3 + b]);
+                break;
+            default:
+                h0 = dir > 0 ? fma2(n1, v0, psi[b]) : add2(psi[b], v0);
+                h1 = dir > 0 ? fma2(n1, v1, psi[3 + b]) : add2(psi[3 + b], v1);
+                break;
+        }
+        const f2 g0 = dir > 0 ? rot2(h0) : nrot2(h0), g1 = dir > 0 ? rot2(h1) : nrot2(h1);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const cx<float> e = dir > 0 ? u[a][b] : u[b][a];
+            const f2 er = dup2(e.re), ei = dup2(e.im);
+            w0[a] = b == 0 ? mul2(er, h0) : fma2(er, h0, w0[a]);
+            w1[a] = b == 0 ? mul2(er, h1) : fma2(er, h1, w1[a]);
+            w0[a] = fma2(ei, g0, w0[a]);
+            w1[a] = fma2(ei, g1, w1[a]);
+        }
+    }
+    const float cl = dir > 0 ? -coeff : coeff;   // of the lower components
+    const f2 c = dup2(coeff), lp = dup2(cl), lm = dup2(-cl), li = pk2(-cl, cl), lni = pk2(cl, -cl);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        out[a] = fma2(c, w0[a], out[a]);
+        out[3 + a] = fma2(c, w1[a], out[3 + a]);
+        // cl e_mu^dag w
+        switch (mu) {
+            case 0:
+                out[6 + a] = fma2(lni, swap2(w1[a]), out[6 + a]);
+                out[9 + a] = fma2(lni, swap2(w0[a]), out[9 + a]);
+                break;
+            case 1:
+                out[6 + a] = fma2(lm, w1[a], out[6 + a]);
+                out[9 + a] = fma2(lp, w0[a], out[9 + a]);
+                break;
+            case 2:
+                out[6 + a] = fma2(lni, swap2(w0[a]), out[6 + a]);
+                out[9 + a] = fma2(li, swap2(w1[a]), out[9 + a]);
+                break;
+            default:
+                out[6 + a] = fma2(lp, w0[a], out[6 + a]);
+                out[9 + a] = fma2(lp, w1[a], out[9 + a]);
+                break;
+        }
+    }
+}
+
 // ------------------------------------------------------------ SAP half sweep
 // One CTA per domain of the given colour, one thread per site of the domain.
 // Computes r = b - D x on the domain (the residual of the SAP listing, needed
@@ -1096,27 +1256,16 @@ __global__ void clover_invert_kernel(Geom g, const void* C64, void* out) {
 // x_mode: 0 = x holds the current iterate everywhere; 1 = x is zero everywhere
 // (r = b, x is only written); 2 = x is zero on the active domains and holds the
 // iterate elsewhere (first odd half sweep after an even sweep from zero).
-// 256-thread FP32/FP16 variant: 128 registers, two CTAs per SM (no spills);
-// the FP64 variant keeps one CTA per SM (it would spill at 128 registers)
-// NR right-hand sides per CTA (NR = 2 for batches, variant 2): thread (slot, l) works on site l
-// for right-hand side NR * (pair index) + slot; both slots read the same domain's links and
-// clover in lockstep, so one domain's operator occupies the SM's L1 instead of two domains'.
-// The body of one CTA: domain k of the given colour, right-hand sides NR * rpair + slot; with
-// DS the NR slots take domains NR * k + slot of right-hand side rpair instead (small domains
-// of a ragged batch, two to a CTA)
-template <class P, int NR, bool DS = false>
+// FP64 domains, and FP32 / FP16 domains of more than 256 sites (sap_pairs_body takes the rest).
+template <class P>
 DEV void sap_half_body(const Geom& g, const Blocking& bk, int colour, int nmr, int x_mode,
                        const void* __restrict__ U, const void* __restrict__ C, const void* __restrict__ b, void* x,
-                       typename P::T kappa, int k0, int rpair, int nrhs) {
+                       typename P::T kappa, int k, int rr) {
     using T = typename P::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int vbp = blockDim.x / NR;
-    const int slot = NR == 1 ? 0 : threadIdx.x / vbp;
-    cx<T>* rsh = reinterpret_cast<cx<T>*>(smem_raw) + (size_t)slot * 12 * vbp;      // [NR][12][vbp]
-    T* red = reinterpret_cast<T*>(reinterpret_cast<cx<T>*>(smem_raw) + (size_t)NR * 12 * vbp) + slot * 192;   // [NR][2][3][32]
-    const int rr = DS ? rpair : NR * rpair + slot;
-    const int k = DS ? NR * k0 + slot : k0;
-    const bool rhs_ok = rr < nrhs && (!DS || k < bk.Vc / 2);
+    const int vbp = blockDim.x;
+    cx<T>* rsh = reinterpret_cast<cx<T>*>(smem_raw);      // [12][vbp]
+    T* red = reinterpret_cast<T*>(rsh + (size_t)12 * vbp);   // [2][3][32]
     const int h0 = bk.C[0] / 2;
     int rest = k / h0;
     int X1 = rest % bk.C[1];
@@ -1126,13 +1275,13 @@ DEV void sap_half_body(const Geom& g, const Blocking& bk, int colour, int nmr, i
     int X0 = 2 * (k % h0) + ((X1 + X2 + X3 + colour) & 1);
     const int Xi = X0 + bk.C[0] * (X1 + bk.C[1] * (X2 + bk.C[2] * X3));
 
-    const int l = threadIdx.x - slot * vbp;
-    const bool active = l < bk.Vb && rhs_ok;
+    const int l = threadIdx.x;
+    const bool active = l < bk.Vb;
     int c[4] = {0, 0, 0, 0}, lc[4] = {0, 0, 0, 0}, s = 0;
     const int lstr[4] = {1, bk.b[0], bk.b[0] * bk.b[1], bk.b[0] * bk.b[1] * bk.b[2]};
     cx<T> r[12], z[12], Ar[12];
-    b = (const char*)b + (rhs_ok ? rr : 0) * spinor_bytes<P>(g.V);
-    x = (char*)x + (rhs_ok ? rr : 0) * spinor_bytes<P>(g.V);
+    b = (const char*)b + rr * spinor_bytes<P>(g.V);
+    x = (char*)x + rr * spinor_bytes<P>(g.V);
     if (active) {
         s = block_site(g, bk, Xi, l, c);
         for (int mu = 0; mu < 4; ++mu) lc[mu] = c[mu] % bk.b[mu];
@@ -1240,16 +1389,191 @@ DEV void sap_half_body(const Geom& g, const Blocking& bk, int colour, int nmr, i
     }
 }
 
-// domain of a CTA: the k-th domain of the given colour; right-hand side group of a batch.
-// rhs_fast: the right-hand side is the fast grid index, so the CTAs of one domain for all
-// right-hand sides run together and share the domain's links and clover in L1/L2
-template <class P, int MAXT, int NR>
-__global__ void __launch_bounds__(MAXT * NR, (MAXT == 256 && NR == 1 && P::id != 0) ? 2 : 1)
+// The half sweep for FP32 arithmetic (FP32 or FP16 storage, domains of at most 256 sites) in packed
+// pairs; NR domains of one right-hand side per CTA (two small domains of a ragged batch)
+template <class P, int NR>
+DEV void sap_pairs_body(const Geom& g, const Blocking& bk, int colour, int nmr, int x_mode,
+                        const void* __restrict__ U, const void* __restrict__ C, const void* __restrict__ b, void* x,
+                        float kappa, int k0, int rr) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int vbp = blockDim.x / NR;
+    const int slot = NR == 1 ? 0 : threadIdx.x / vbp;
+    float4* rsh = reinterpret_cast<float4*>(smem_raw) + (size_t)slot * 6 * vbp;   // [NR][6][vbp]
+    float4* red = reinterpret_cast<float4*>(smem_raw) + (size_t)6 * blockDim.x;    // [2][warps]
+    const int k = NR * k0 + slot;
+    auto sync = [&]() {   // the slots run independently
+        if constexpr (NR == 1) __syncthreads();
+        else asm volatile("bar.sync %0, %1;" ::"r"(slot + 1), "r"(vbp) : "memory");
+    };
+    const int l = threadIdx.x - slot * vbp, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nw = (vbp + 31) >> 5, nwt = blockDim.x >> 5;
+    const bool active = l < bk.Vb && k < bk.Vc / 2;
+    int c[4] = {0, 0, 0, 0}, lc[4] = {0, 0, 0, 0}, s = 0;
+    const int lstr[4] = {1, bk.b[0], bk.b[0] * bk.b[1], bk.b[0] * bk.b[1] * bk.b[2]};
+    f2 r[12], z[12], Ar[12];
+    b = (const char*)b + rr * spinor_bytes<P>(g.V);
+    x = (char*)x + rr * spinor_bytes<P>(g.V);
+    if (active) {
+        const int h0 = bk.C[0] / 2;
+        int rest = k / h0;
+        const int X1 = rest % bk.C[1];
+        rest /= bk.C[1];
+        const int X2 = rest % bk.C[2], X3 = rest / bk.C[2];
+        const int X0 = 2 * (k % h0) + ((X1 + X2 + X3 + colour) & 1);
+        s = block_site(g, bk, X0 + bk.C[0] * (X1 + bk.C[1] * (X2 + bk.C[2] * X3)), l, c);
+#pragma unroll
+        for (int mu = 0; mu < 4; ++mu) lc[mu] = c[mu] % bk.b[mu];
+        load_pairs<P>(b, g.V, s, r);
+        if (x_mode != 1) {
+            // r = b - D x at this site; with x_mode 2 only hops from outside the domain contribute
+            f2 psi[12];
+#pragma unroll
+            for (int q = 0; q < 12; ++q) Ar[q] = dup2(0.f);
+            if (x_mode == 0) {
+                load_pairs<P>(x, g.V, s, psi);
+                float pr[36];
+                CloverIO<P>::load_block(C, g.V, s, 0, pr);
+                clover_pairs(pr, psi, Ar);
+                CloverIO<P>::load_block(C, g.V, s, 1, pr);
+                clover_pairs(pr, psi + 6, Ar + 6);
+            }
+#pragma unroll
+            for (int mu = 0; mu < 4; ++mu) {
+                float ph;
+                cx<float> u[3][3];
+                if (x_mode == 0 || lc[mu] == bk.b[mu] - 1) {
+                    int n = neighbour(g, s, c, mu, +1, ph);
+                    load_pairs<P>(x, g.V, n, psi);
+                    GaugeIO<P>::load(U, g.V, mu, s, u);
+                    hop_pairs(Ar, psi, u, mu, +1, -kappa * ph);
+                }
+                if (x_mode == 0 || lc[mu] == 0) {
+                    int n = neighbour(g, s, c, mu, -1, ph);
+                    load_pairs<P>(x, g.V, n, psi);
+                    GaugeIO<P>::load(U, g.V, mu, n, u);
+                    hop_pairs(Ar, psi, u, mu, -1, -kappa * ph);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 12; ++q) r[q] = fma2(dup2(-1.f), Ar[q], r[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < 12; ++q) z[q] = dup2(0.f);
+        tile_put(rsh, vbp, l, r);
+    }
+    for (int it = 0; it < nmr; ++it) {
+        sync();
+        float part[4] = {0.f, 0.f, 0.f, 0.f};
+        if (active) {
+            float pr[36];
+            CloverIO<P>::load_block(C, g.V, s, 0, pr);
+            clover_pairs(pr, r, Ar);
+            CloverIO<P>::load_block(C, g.V, s, 1, pr);
+            clover_pairs(pr, r + 6, Ar + 6);
+#pragma unroll
+            for (int mu = 0; mu < 4; ++mu) {
+                cx<float> u[3][3];
+                f2 psi[12];
+                if (lc[mu] != bk.b[mu] - 1) {
+                    tile_get(rsh, vbp, l + lstr[mu], psi);
+                    GaugeIO<P>::load(U, g.V, mu, s, u);
+                    hop_pairs(Ar, psi, u, mu, +1, -kappa);
+                }
+                if (lc[mu] != 0) {
+                    tile_get(rsh, vbp, l - lstr[mu], psi);
+                    GaugeIO<P>::load(U, g.V, mu, s - g.stride[mu], u);
+                    hop_pairs(Ar, psi, u, mu, -1, -kappa);
+                }
+            }
+            // <Ar, r> and |Ar|^2, the two halves of each pair summed at the end
+            f2 p0 = dup2(0.f), p1 = p0, p2 = p0;
+#pragma unroll
+            for (int q = 0; q < 12; ++q) {
+                p0 = fma2(Ar[q], r[q], p0);
+                p1 = fma2(Ar[q], swap2(r[q]), p1);
+                p2 = fma2(Ar[q], Ar[q], p2);
+            }
+            float a0, a1;
+            unpk2(p0, a0, a1);
+            part[0] = a0 + a1;
+            unpk2(p1, a0, a1);
+            part[1] = a0 - a1;
+            unpk2(p2, a0, a1);
+            part[2] = a0 + a1;
+        }
+        // one-barrier reduction into buffer (it & 1): the loop's top barrier keeps the other
+        // buffer's readers of the previous step apart from its next writers
+        const float tw = transposed_warp_sum<4>(part, lane);
+        if ((lane & 7) == 0) reinterpret_cast<float*>(red + (it & 1) * nwt + warp)[transposed_index<4>(lane)] = tw;
+        sync();
+        float4 tot = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int w = 0; w < nw; ++w) {
+            const float4 t = red[(it & 1) * nwt + slot * nw + w];
+            tot.x += t.x;
+            tot.y += t.y;
+            tot.z += t.z;
+        }
+        cx<float> alpha = czero<float>();
+        if (tot.z > 0.f) alpha = {tot.x / tot.z, tot.y / tot.z};
+        if (active) {
+            const f2 ar = dup2(alpha.re), ai = pk2(-alpha.im, alpha.im);
+#pragma unroll
+            for (int q = 0; q < 12; ++q) {
+                z[q] = fma2(ar, r[q], z[q]);
+                z[q] = fma2(ai, swap2(r[q]), z[q]);
+            }
+            if (it + 1 < nmr) {   // the last step's residual is not needed
+                const f2 nr = dup2(-alpha.re), ni = pk2(alpha.im, -alpha.im);
+#pragma unroll
+                for (int q = 0; q < 12; ++q) {
+                    r[q] = fma2(nr, Ar[q], r[q]);
+                    r[q] = fma2(ni, swap2(Ar[q]), r[q]);
+                }
+                tile_put(rsh, vbp, l, r);
+            }
+        }
+    }
+    if (active) {
+        cx<float> o[12];
+        if (x_mode == 0) {
+            f2 x0[12];
+            load_pairs<P>(x, g.V, s, x0);
+#pragma unroll
+            for (int q = 0; q < 12; ++q) z[q] = add2(z[q], x0[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < 12; ++q) unpk2(z[q], o[q].re, o[q].im);
+        SpinorIO<P>::store(x, g.V, s, o);
+    }
+}
+// 128 registers, two CTAs of 256 threads per SM.  24^3 x 48, 4^4 domains, per right-hand side and
+// SAP application: 1.61 -> 1.55 ms in a batch of twelve, 2.26 -> 2.07 ms alone (scalar -> packed;
+// 486 -> 360 M warp instructions per half sweep of four).  The FP32 pipe is busy half of the time
+// in every form tried: a step's multiply-adds, loads and reduction follow one another behind
+// barriers, and 16 warps overlap them only in part.  As fast or slower: the operator in shared
+// memory (one CTA of two right-hand sides per SM, 1.59 ms; alone 2.29), two right-hand sides per
+// CTA through L1 (1.68 ms), the operator in registers at 8 warps per SM (1.75 ms in a batch of
+// four, 1.61 here).
+template <class P>
+__global__ void __launch_bounds__(256, 2)
+    sap_pairs_kernel(Geom g, Blocking bk, int colour, int nmr, int x_mode, const void* __restrict__ U,
+                     const void* __restrict__ C, const void* __restrict__ b, void* x, float kappa, int rhs_fast) {
+    sap_pairs_body<P, 1>(g, bk, colour, nmr, x_mode, U, C, b, x, kappa, rhs_fast ? blockIdx.y : blockIdx.x,
+                         rhs_fast ? blockIdx.x : blockIdx.y);
+}
+HD constexpr size_t sap_pairs_smem(int threads) { return (size_t)threads * 96 + 2 * 8 * 16; }
+
+// domain of a CTA: the k-th domain of the given colour.  rhs_fast: the right-hand side is the fast
+// grid index, so the CTAs of one domain for all right-hand sides run together and share the
+// domain's links and clover in L2.  One CTA per SM for 256 threads of FP64 (it would spill at
+// 128 registers).
+template <class P, int MAXT>
+__global__ void __launch_bounds__(MAXT, 1)
     sap_half_kernel(Geom g, Blocking bk, int colour, int nmr, int x_mode, const void* __restrict__ U,
                     const void* __restrict__ C, const void* __restrict__ b, void* x, typename P::T kappa,
-                    int rhs_fast, int nrhs) {
-    sap_half_body<P, NR>(g, bk, colour, nmr, x_mode, U, C, b, x, kappa, rhs_fast ? blockIdx.y : blockIdx.x,
-                         rhs_fast ? blockIdx.x : blockIdx.y, nrhs);
+                    int rhs_fast) {
+    sap_half_body<P>(g, bk, colour, nmr, x_mode, U, C, b, x, kappa, rhs_fast ? blockIdx.y : blockIdx.x,
+                     rhs_fast ? blockIdx.x : blockIdx.y);
 }
 
 // the half sweep for every problem of a ragged batch in one launch: CTA ranges per problem
@@ -1262,8 +1586,8 @@ __global__ void __launch_bounds__(256, 2)
     int p, bx, gx;
     ragged_locate(off, np, p, bx, gx);
     const RaggedDev& q = d[p];
-    if (q.sap_nr == 2) sap_half_body<P32, 2, true>(q.g, q.bk, colour, nmr, 0, q.U32, q.C32, q.f32, q.z, q.kappa32, bx, 0, 1);
-    else sap_half_body<P32, 1>(q.g, q.bk, colour, nmr, 0, q.U32, q.C32, q.f32, q.z, q.kappa32, bx, 0, 1);
+    if (q.sap_nr == 2) sap_pairs_body<P32, 2>(q.g, q.bk, colour, nmr, 0, q.U32, q.C32, q.f32, q.z, q.kappa32, bx, 0);
+    else sap_pairs_body<P32, 1>(q.g, q.bk, colour, nmr, 0, q.U32, q.C32, q.f32, q.z, q.kappa32, bx, 0);
 }
 
 // ------------------------------------------------------------ SAP half sweep, even-odd domain solves
@@ -1450,39 +1774,11 @@ __global__ void __launch_bounds__(128, P::id == 0 ? 2 : 4)
     }
 }
 
-// ------------------------------------------------------------ SAP half sweep, staged operator
-// Same algorithm as sap_half_kernel, but the domain's own forward links and
-// clover are copied to shared memory once, so the nmr minimal-residual steps
-// read the operator only from shared memory; the block reduction uses one
-// barrier per step (double-buffered partials).  FP32 and FP16 storage.
+// ------------------------------------------------------------ SAP half sweep, FP16 copy of the operator
+// (sap_variant 3) FP32 vectors; the domain's own forward links and clover are copied to shared
+// memory once from the FP16 fields, so the nmr minimal-residual steps read the operator only from
+// shared memory; the block reduction uses one barrier per step (double-buffered partials).
 template <class P> struct Staged;
-template <> struct Staged<P32> {
-    using LC = float4;   // link chunk: 3 per link
-    using CC = float4;   // clover chunk: 18 per site
-    static constexpr int kLinkChunks = 3, kCloverChunks = 18;
-    DEV static void link(const LC* sl, int vbp, int mu, int l, cx<float> u[3][3]) {
-        const LC* p = sl + (size_t)mu * 3 * vbp;
-        float4 a = p[l], b = p[vbp + l], c = p[2 * vbp + l];
-        u[0][0] = {a.x, a.y};
-        u[0][1] = {a.z, a.w};
-        u[0][2] = {b.x, b.y};
-        u[1][0] = {b.z, b.w};
-        u[1][1] = {c.x, c.y};
-        u[1][2] = {c.z, c.w};
-        reconstruct_row2(u);
-    }
-    DEV static void clover_block(const CC* sc, int vbp, int l, int b, float pr[36]) {
-        const CC* p = sc + (size_t)9 * b * vbp;
-#pragma unroll
-        for (int q = 0; q < 9; ++q) {
-            float4 t = p[q * vbp + l];
-            pr[4 * q] = t.x;
-            pr[4 * q + 1] = t.y;
-            pr[4 * q + 2] = t.z;
-            pr[4 * q + 3] = t.w;
-        }
-    }
-};
 template <> struct Staged<P16> {
     using LC = uint2;   // 3 per link
     using CC = uint4;   // 9 per site
@@ -1714,43 +2010,38 @@ cudaError_t sap_half_staged_impl(const GeomH& gh, const BlockH& bh, int colour, 
 }
 
 template <class P>
+cudaError_t sap_pairs_impl(const GeomH& gh, const BlockH& bh, int colour, int nmr, int x_mode, const void* U,
+                           const void* C, const void* b, void* x, double kappa, int nrhs, cudaStream_t st) {
+    Geom g = make_geom(gh);
+    const Blocking bk = make_blocking(gh, bh);
+    const int threads = (bk.Vb + 31) / 32 * 32, ndom = bk.Vc / 2;
+    if (threads > 256) return cudaErrorInvalidValue;
+    // right-hand side as the fast grid index when the domains fit the y dimension
+    const int fast = nrhs > 1 && ndom <= 65535;
+    const dim3 grid = fast ? dim3(nrhs, ndom) : dim3(ndom, nrhs);
+    (note_launch(), sap_pairs_kernel<P><<<grid, threads, sap_pairs_smem(threads), st>>>(g, bk, colour, nmr, x_mode, U, C,
+                                                                                       b, x, (float)kappa, fast));
+    return cudaGetLastError();
+}
+
+template <class P>
 cudaError_t sap_half_impl(const GeomH& gh, const BlockH& bh, int colour, int nmr, int x_mode, const void* U,
-                          const void* C, const void* b, void* x, double kappa, int nrhs, cudaStream_t st,
-                          bool pair = false) {
+                          const void* C, const void* b, void* x, double kappa, int nrhs, cudaStream_t st) {
     Geom g = make_geom(gh);
     Blocking bk = make_blocking(gh, bh);
     int threads = (bk.Vb + 31) / 32 * 32;
     if (threads > 512) return cudaErrorInvalidValue;
-    // two right-hand sides per CTA (variant 2, batches, FP32/FP16, blocks of <= 256 sites)
-    const int nr = (pair && nrhs > 1 && threads <= 256 && P::id != 0) ? 2 : 1;
-    size_t smem = (size_t)nr * 12 * threads * sizeof(cx<typename P::T>) + nr * 2 * 3 * 32 * sizeof(typename P::T);
+    size_t smem = (size_t)12 * threads * sizeof(cx<typename P::T>) + 2 * 3 * 32 * sizeof(typename P::T);
     int ndom = bk.Vc / 2;
-    const int ngrp = (nrhs + nr - 1) / nr;
     // right-hand side as the fast grid index when the domains fit the y dimension
-    const int fast = ngrp > 1 && ndom <= 65535;
-    const dim3 grid = fast ? dim3(ngrp, ndom) : dim3(ndom, ngrp);
+    const int fast = nrhs > 1 && ndom <= 65535;
+    const dim3 grid = fast ? dim3(nrhs, ndom) : dim3(ndom, nrhs);
     const typename P::T kp = (typename P::T)kappa;
-    if constexpr (P::id != 0) {
-        if (nr == 2) {
-            auto fn = sap_half_kernel<P, 256, 2>;
-            cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-            (note_launch(), fn<<<grid, 2 * threads, smem, st>>>(g, bk, colour, nmr, x_mode, U, C, b, x, kp, fast,
-                                                                 nrhs));
-            return cudaGetLastError();
-        }
-    }
-    if (threads <= 256) {
-        auto fn = sap_half_kernel<P, 256, 1>;
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        (note_launch(), fn<<<grid, threads, smem, st>>>(g, bk, colour, nmr, x_mode, U, C, b, x, kp, fast, nrhs));
-    } else {
-        auto fn = sap_half_kernel<P, 512, 1>;
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        (note_launch(), fn<<<grid, threads, smem, st>>>(g, bk, colour, nmr, x_mode, U, C, b, x, kp, fast, nrhs));
-    }
+    // FP32 / FP16 domains of at most 256 sites run sap_pairs_kernel
+    auto fn = P::id == 0 && threads <= 256 ? sap_half_kernel<P, P::id == 0 ? 256 : 512> : sap_half_kernel<P, 512>;
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    (note_launch(), fn<<<grid, threads, smem, st>>>(g, bk, colour, nmr, x_mode, U, C, b, x, kp, fast));
     return cudaGetLastError();
 }
 
@@ -2049,17 +2340,14 @@ cudaError_t launch_clover_invert(int prec, const GeomH& gh, const void* C64, voi
     return cudaGetLastError();
 }
 
-cudaError_t launch_sap_half_variant(int variant, int prec, const GeomH& g, const BlockH& bk, int colour, int nmr,
-                                    int x_mode, const void* U, const void* C, const void* b, void* x, double kappa,
-                                    int nrhs, cudaStream_t st) {
-    if (variant == 1 && prec == 1)
-        return sap_half_staged_impl<P32>(g, bk, colour, nmr, x_mode, U, C, b, x, kappa, nrhs, st);
-    if (variant == 1 && prec == 2)
-        return sap_half_staged_impl<P16>(g, bk, colour, nmr, x_mode, U, C, b, x, kappa, nrhs, st);
-    const bool pair = variant == 2;
-    if (prec == 0) return sap_half_impl<P64>(g, bk, colour, nmr, x_mode, U, C, b, x, kappa, nrhs, st, pair);
-    if (prec == 1) return sap_half_impl<P32>(g, bk, colour, nmr, x_mode, U, C, b, x, kappa, nrhs, st, pair);
-    return sap_half_impl<P16>(g, bk, colour, nmr, x_mode, U, C, b, x, kappa, nrhs, st, pair);
+cudaError_t launch_sap_half(int prec, const GeomH& g, const BlockH& bk, int colour, int nmr, int x_mode, const void* U,
+                            const void* C, const void* b, void* x, double kappa, int nrhs, cudaStream_t st) {
+    if (sap_staged_supported(prec, bk))
+        return prec == 1 ? sap_pairs_impl<P32>(g, bk, colour, nmr, x_mode, U, C, b, x, kappa, nrhs, st)
+                         : sap_pairs_impl<P16>(g, bk, colour, nmr, x_mode, U, C, b, x, kappa, nrhs, st);
+    if (prec == 0) return sap_half_impl<P64>(g, bk, colour, nmr, x_mode, U, C, b, x, kappa, nrhs, st);
+    if (prec == 1) return sap_half_impl<P32>(g, bk, colour, nmr, x_mode, U, C, b, x, kappa, nrhs, st);
+    return sap_half_impl<P16>(g, bk, colour, nmr, x_mode, U, C, b, x, kappa, nrhs, st);
 }
 cudaError_t launch_sap_half_staged16(const GeomH& g, const BlockH& bk, int colour, int nmr, int x_mode,
                                      const void* U32, const void* C32, const void* U16, const void* C16,
@@ -2069,12 +2357,6 @@ cudaError_t launch_sap_half_staged16(const GeomH& g, const BlockH& bk, int colou
 bool sap_staged_supported(int prec, const BlockH& bk) {
     int vb = bk.b[0] * bk.b[1] * bk.b[2] * bk.b[3];
     return (prec == 1 || prec == 2) && vb <= 256;
-}
-cudaError_t launch_sap_half(int prec, const GeomH& g, const BlockH& bk, int colour, int nmr, int x_mode, const void* U,
-                            const void* C, const void* b, void* x, double kappa, cudaStream_t st) {
-    if (prec == 0) return sap_half_impl<P64>(g, bk, colour, nmr, x_mode, U, C, b, x, kappa, 1, st);
-    if (prec == 1) return sap_half_impl<P32>(g, bk, colour, nmr, x_mode, U, C, b, x, kappa, 1, st);
-    return sap_half_impl<P16>(g, bk, colour, nmr, x_mode, U, C, b, x, kappa, 1, st);
 }
 
 // ---------------------------------------------------------------- ragged batches
@@ -2153,7 +2435,7 @@ cudaError_t launch_sap_half_ragged(const void* d, const int* off, int np, int ct
                                    cudaStream_t st) {
     const int threads = ragged_sap_threads(max_vb);
     if (max_vb > 256 || ctas < 1) return cudaErrorInvalidValue;
-    const size_t smem = (size_t)12 * threads * sizeof(cx<float>) + 2 * 2 * 3 * 32 * sizeof(float);
+    const size_t smem = sap_pairs_smem(threads);
     (note_launch(), sap_half_ragged_kernel<<<ctas, threads, smem, st>>>((const RaggedDev*)d, off, np, colour, nmr));
     return cudaGetLastError();
 }

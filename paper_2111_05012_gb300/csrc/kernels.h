@@ -82,13 +82,9 @@ cudaError_t launch_spinor_axpy_mixed(const GeomH& g, int k, const double2* c, co
 //   r = b - D x on the domain, z = MR_nmr(D_SAP, r), x += z
 //   x_mode 0: x holds the iterate; 1: x is zero everywhere; 2: x is zero on the active domains
 cudaError_t launch_sap_half(int prec, const GeomH& g, const BlockH& bk, int colour, int nmr, int x_mode,
-                            const void* U, const void* C, const void* b, void* x, double kappa, cudaStream_t s);
-
-// variant 0: operator read from global memory in every MR step (all precisions);
-// variant 1: domain operator staged in shared memory (FP32 / FP16, blocks <= 256 sites)
-cudaError_t launch_sap_half_variant(int variant, int prec, const GeomH& g, const BlockH& bk, int colour, int nmr,
-                                    int x_mode, const void* U, const void* C, const void* b, void* x, double kappa,
-                                    int nrhs, cudaStream_t s);
+                            const void* U, const void* C, const void* b, void* x, double kappa, int nrhs,
+                            cudaStream_t s);
+// FP32 / FP16 domains of at most 256 sites (packed-pair kernel; staged FP16 operator for FP32)
 bool sap_staged_supported(int prec, const BlockH& bk);
 // variant 3 (FP32 smoother, blocks <= 256 sites): the domain operator staged in shared memory from
 // its FP16 copy (U16, C16: prec-2 fields), FP32 arithmetic and vectors; the residual b - D x uses
