@@ -124,24 +124,19 @@ struct Reducer {
         }
         return AMG_OK;
     }
-    // for r < nb: k dots <a_r[j], b_r> (a_r = a + r * stride entries, likewise b), one
-    // synchronisation for the batch; out[r * k + j]; k * nb <= 20 * capacity
-    amg_status batch_dots(int prec, int nb, int k, const void* const* a, const void* b, size_t stride, size_t n,
-                          cplx* out, cudaStream_t s) {
-        const size_t eb = prec == 0 ? 16 : 8;
-        std::vector<const void*> ar(k);
-        for (int r = 0; r < nb; ++r) {
-            for (int j = 0; j < k; ++j) ar[j] = (const char*)a[j] + r * stride * eb;
-            CK(launch_multi_dot(prec, k, ar.data(), (const char*)b + r * stride * eb, n,
-                                dpart.as<double2>() + (size_t)r * k * grid, s));
-        }
-        CK(cudaMemcpyAsync(hpart, dpart.p, sizeof(double2) * grid * k * nb, cudaMemcpyDeviceToHost, s));
+    // FP32 batches of nb vectors (right-hand side r at r * n): out[r * nq + q] = <a_q, b> for the k
+    // vectors a, or the upper triangle <a_p, a_q> (p <= q) if b is null; one launch and one
+    // synchronisation for the batch
+    amg_status batch_dots(int nb, int k, void* const* a, const void* b, size_t n, cplx* out, cudaStream_t s) {
+        const int nq = (b ? k : k * (k + 1) / 2) * nb, ctas = batch_ctas(n);
+        CK(launch_batch_dot(k, a, b, n, nb, dpart.as<double2>(), s));
+        CK(cudaMemcpyAsync(hpart, dpart.p, sizeof(double2) * ctas * nq, cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
-        for (int j = 0; j < k * nb; ++j) {
+        for (int j = 0; j < nq; ++j) {
             double re = 0, im = 0;
-            for (int q = 0; q < grid; ++q) {
-                re += hpart[j * grid + q].x;
-                im += hpart[j * grid + q].y;
+            for (int q = 0; q < ctas; ++q) {
+                re += hpart[(size_t)j * ctas + q].x;
+                im += hpart[(size_t)j * ctas + q].y;
             }
             out[j] = cplx(re, im);
         }
@@ -466,10 +461,15 @@ amg_status coarse_bicgstab_tc(amg_hierarchy* h, int l, const void* b, void* x, i
         R[j] = L.tcw[1 + j].p;
         U[j] = L.tcw[2 + ell + j].p;
     }
-    auto F = [&](const void* base, int r) { return (char*)base + r * vb; };
-    const double2 one = make_double2(1, 0);
     Reducer& red = h->red;
-    TRY(red.init(std::max(nb, 2)));
+    TRY(red.init(std::max(nb, 2)));   // 20 x 304 partials per right-hand side; the largest use is 15 x 152
+    std::vector<double2> coef((size_t)nb * 15);   // [right-hand side][3][5]
+    auto cf = [&](int r, int q, int k) -> double2& { return coef[((size_t)r * 3 + q) * 5 + k]; };
+    auto active = [&](const std::vector<char>& a) {
+        unsigned m = 0;
+        for (int r = 0; r < nb; ++r) m |= (a[r] ? 1u : 0u) << r;
+        return m;
+    };
     CK(cudaMemsetAsync(x, 0, vb * nb, s));
     CK(cudaMemsetAsync(U[0], 0, vb * nb, s));
     CK(cudaMemcpyAsync(R[0], b, vb * nb, cudaMemcpyDeviceToDevice, s));
@@ -486,8 +486,8 @@ amg_status coarse_bicgstab_tc(amg_hierarchy* h, int l, const void* b, void* x, i
         // |R_0|^2 and <r~, R_0> per right-hand side
         std::vector<cplx> q(2 * nb);
         {
-            const void* a2[2] = {R[0], rt};
-            TRY(red.batch_dots(1, nb, 2, a2, R[0], n, n, q.data(), s));
+            void* a2[2] = {R[0], rt};
+            TRY(red.batch_dots(nb, 2, a2, R[0], n, q.data(), s));
         }
         bool any = false;
         for (int r = 0; r < nb; ++r) {
@@ -509,56 +509,57 @@ amg_status coarse_bicgstab_tc(amg_hierarchy* h, int l, const void* b, void* x, i
                 if (!act[r]) continue;
                 const cplx beta = alpha[r] * rho1[r] / rho0[r];
                 rho0[r] = rho1[r];
-                for (int i = 0; i <= j; ++i) CK(launch_axpby(1, one, F(R[i], r), d2(-beta), F(U[i], r), n, s));
+                cf(r, 0, 0) = d2(-beta);
             }
+            CK(launch_batch_update(0, ell, R.data(), U.data(), x, coef.data(), active(act), j, n, nb, s));
             TRY(stencil(U[j], U[j + 1]));
             std::vector<cplx> gam(nb);
             {
-                const void* a1[1] = {rt};
-                TRY(red.batch_dots(1, nb, 1, a1, U[j + 1], n, n, gam.data(), s));
+                void* a1[1] = {rt};
+                TRY(red.batch_dots(nb, 1, a1, U[j + 1], n, gam.data(), s));
             }
             for (int r = 0; r < nb; ++r) {
                 if (!act[r]) continue;
                 alpha[r] = rho0[r] / gam[r];
                 if (!std::isfinite(alpha[r].real()) || !std::isfinite(alpha[r].imag()))
                     return fail(AMG_NAN, "coarse solver: BiCGStab breakdown");
-                for (int i = 0; i <= j; ++i) CK(launch_axpby(1, d2(-alpha[r]), F(U[i + 1], r), one, F(R[i], r), n, s));
-                CK(launch_axpby(1, d2(alpha[r]), F(U[0], r), one, F(x, r), n, s));
+                cf(r, 0, 0) = d2(-alpha[r]);
+                cf(r, 1, 0) = d2(alpha[r]);
             }
+            CK(launch_batch_update(1, ell, R.data(), U.data(), x, coef.data(), active(act), j, n, nb, s));
             TRY(stencil(R[j], R[j + 1]));
             if (j + 1 < ell) {
                 std::vector<cplx> r1(nb);
-                const void* a1[1] = {rt};
-                TRY(red.batch_dots(1, nb, 1, a1, R[j + 1], n, n, r1.data(), s));
+                void* a1[1] = {rt};
+                TRY(red.batch_dots(nb, 1, a1, R[j + 1], n, r1.data(), s));
                 for (int r = 0; r < nb; ++r)
                     if (act[r]) rho1[r] = r1[r];
             }
         }
         // Gram matrices G_pq = <R_p, R_q> of every right-hand side, then the minimal-residual part
-        std::vector<cplx> gm((size_t)nb * (ell + 1) * (ell + 1));
-        for (int qq = 0; qq <= ell; ++qq) {
-            std::vector<cplx> row((size_t)nb * (ell + 1));
-            std::vector<const void*> al(R.begin(), R.end());
-            TRY(red.batch_dots(1, nb, ell + 1, al.data(), R[qq], n, n, row.data(), s));
-            for (int r = 0; r < nb; ++r)
-                for (int p = 0; p <= ell; ++p) gm[((size_t)r * (ell + 1) + p) * (ell + 1) + qq] = row[r * (ell + 1) + p];
-        }
+        const int npair = (ell + 1) * (ell + 2) / 2;
+        std::vector<cplx> gm((size_t)nb * npair);
+        TRY(red.batch_dots(nb, ell + 1, R.data(), nullptr, n, gm.data(), s));
         for (int r = 0; r < nb; ++r) {
             if (!act[r]) continue;
             std::vector<std::vector<cplx>> G(ell + 1, std::vector<cplx>(ell + 1));
+            const cplx* gr = gm.data() + (size_t)r * npair;
             for (int p = 0; p <= ell; ++p)
-                for (int qq = 0; qq <= ell; ++qq) G[p][qq] = gm[((size_t)r * (ell + 1) + p) * (ell + 1) + qq];
+                for (int qq = p; qq <= ell; ++qq) {
+                    G[p][qq] = *gr++;
+                    G[qq][p] = std::conj(G[p][qq]);
+                }
             std::vector<cplx> cxv, crv, cgv;
             if (!bicgstab_mr_coefficients(G, ell, cxv, crv, cgv))
                 return fail(AMG_NAN, "coarse solver: BiCGStab breakdown");
             omega[r] = cgv[ell];
-            CK(launch_axpby(1, d2(cxv[0]), F(R[0], r), one, F(x, r), n, s));
-            for (int k = 1; k <= ell; ++k) {
-                CK(launch_axpby(1, d2(cxv[k]), F(R[k], r), one, F(x, r), n, s));
-                CK(launch_axpby(1, d2(-crv[k]), F(R[k], r), one, F(R[0], r), n, s));
-                CK(launch_axpby(1, d2(-cgv[k]), F(U[k], r), one, F(U[0], r), n, s));
+            for (int k = 0; k <= ell; ++k) {
+                cf(r, 0, k) = d2(cxv[k]);
+                cf(r, 1, k) = k ? d2(-crv[k]) : make_double2(0, 0);
+                cf(r, 2, k) = k ? d2(-cgv[k]) : make_double2(0, 0);
             }
         }
+        CK(launch_batch_update(2, ell, R.data(), U.data(), x, coef.data(), active(act), ell, n, nb, s));
     }
     int terr = 0;
     CK(cudaMemcpyAsync(&terr, L.tcerr.p, sizeof(int), cudaMemcpyDeviceToHost, s));

@@ -214,7 +214,21 @@ template <typename V>
 DEV void norm2_body(const V* __restrict__ a, size_t n, double* partials, int bx, int gx) {
     __shared__ double red[32];
     double acc = 0;
-    for (size_t i = bx * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gx * blockDim.x) {
+    // four loads in flight (the grid is two CTAs per SM; one load at a time left HBM at a third of
+    // its rate: 58 -> 33 us for 8 M FP64 entries), added in the same order
+    const size_t step = (size_t)gx * blockDim.x;
+    size_t i = bx * (size_t)blockDim.x + threadIdx.x;
+    for (; i + 3 * step < n; i += 4 * step) {
+        V x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = a[i + u * step];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            acc = fma((double)x[u].x, (double)x[u].x, acc);
+            acc = fma((double)x[u].y, (double)x[u].y, acc);
+        }
+    }
+    for (; i < n; i += step) {
         V x = a[i];
         acc = fma((double)x.x, (double)x.x, acc);
         acc = fma((double)x.y, (double)x.y, acc);
@@ -266,7 +280,21 @@ DEV void normalise_body(const double* src, double* hn, const V* __restrict__ x, 
     }
     __syncthreads();
     const T a = (T)s_inv;
-    for (size_t i = bx * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gx * blockDim.x) {
+    // four loads in flight, as in norm2_body (71 -> 44 us for 8 M FP64 entries)
+    const size_t step = (size_t)gx * blockDim.x;
+    size_t i = bx * (size_t)blockDim.x + threadIdx.x;
+    for (; i + 3 * step < n; i += 4 * step) {
+        V v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = x[i + u * step];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            v[u].x *= a;
+            v[u].y *= a;
+            y[i + u * step] = v[u];
+        }
+    }
+    for (; i < n; i += step) {
         V v = x[i];
         v.x *= a;
         v.y *= a;
@@ -309,6 +337,114 @@ __global__ void multi_axpy_kernel(int k, CoefList c, PtrList x, V* y, size_t n) 
         o.y = im;
         y[i] = o;
     }
+}
+
+// ---- lockstep coarse solve: a batch of FP32 vectors, right-hand side r at r * n, in one launch
+// per update or reduction (one launch per right-hand side and vector was 180 per BiCGStab(2)
+// cycle of twelve, 4 us each).  blockIdx.y: the right-hand side; the active ones in a bit mask.
+constexpr int kBatchCoef = 5;
+struct BatchVecs {
+    float2* v[10];
+};
+struct BatchCoefs {
+    float2 c[16][3][kBatchCoef];
+    unsigned active;
+};
+// dots <a_p, b> (FP64) for p < k: part[(r * k + p) * gridDim.x + cta]; with GRAM all pairs
+// <a_p, a_q>, p <= q, in the order (0,0) (0,1) .. (0,k-1) (1,1) ..
+template <int K, bool GRAM>
+__global__ void __launch_bounds__(kBT) batch_dot_kernel(BatchVecs a, const float2* __restrict__ b, size_t n,
+                                                        double2* part) {
+    constexpr int NQ = GRAM ? K * (K + 1) / 2 : K;
+    __shared__ double red[2 * NQ * (kBT / 32)];
+    const size_t r = blockIdx.y;
+    double acc[2 * NQ];
+#pragma unroll
+    for (int q = 0; q < 2 * NQ; ++q) acc[q] = 0.0;
+    auto mac = [&](int q, float2 x, float2 y) {   // conj(x) y
+        acc[2 * q] = fma((double)x.x, (double)y.x, acc[2 * q]);
+        acc[2 * q] = fma((double)x.y, (double)y.y, acc[2 * q]);
+        acc[2 * q + 1] = fma((double)x.x, (double)y.y, acc[2 * q + 1]);
+        acc[2 * q + 1] = fma(-(double)x.y, (double)y.x, acc[2 * q + 1]);
+    };
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        float2 x[K];
+#pragma unroll
+        for (int p = 0; p < K; ++p) x[p] = a.v[p][r * n + i];
+        if constexpr (GRAM) {
+            int q = 0;
+#pragma unroll
+            for (int p = 0; p < K; ++p)
+#pragma unroll
+                for (int t = p; t < K; ++t) mac(q++, x[p], x[t]);
+        } else {
+            const float2 y = b[r * n + i];
+#pragma unroll
+            for (int p = 0; p < K; ++p) mac(p, x[p], y);
+        }
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int q = 0; q < 2 * NQ; ++q) {
+        const double v = warp_sum(acc[q]);
+        if (lane == 0) red[q * (kBT / 32) + warp] = v;
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q < NQ; q += kBT) {
+        double re = 0, im = 0;
+        for (int w = 0; w < kBT / 32; ++w) {
+            re += red[2 * q * (kBT / 32) + w];
+            im += red[(2 * q + 1) * (kBT / 32) + w];
+        }
+        part[(r * NQ + q) * gridDim.x + blockIdx.x] = make_double2(re, im);
+    }
+}
+DEV float2 cmac(float2 y, float2 c, float2 x) {
+    y.x = fmaf(c.x, x.x, y.x);
+    y.x = fmaf(-c.y, x.y, y.x);
+    y.y = fmaf(c.x, x.y, y.y);
+    y.y = fmaf(c.y, x.x, y.y);
+    return y;
+}
+// MODE 0: U_i = R_i + c[0] U_i, i <= j.  MODE 1: R_i += c[0] U_{i+1}, i <= j, and x += c[1] U_0.
+// MODE 2: x += sum_k c[0][k] R_k, R_0 += sum_k c[1][k] R_k, U_0 += sum_k c[2][k] U_k, k = 0 .. j
+// (x and R_0 from the old R_0).  v: R_0 .. R_4, U_0 .. U_4.
+template <int MODE>
+__global__ void __launch_bounds__(kBT) batch_update_kernel(BatchVecs v, float2* x, BatchCoefs co, int j, size_t n) {
+    const int r = blockIdx.y;
+    if (!(co.active >> r & 1)) return;
+    const float2(*c)[kBatchCoef] = co.c[r];
+    float2* const* R = v.v;
+    float2* const* U = v.v + 5;
+    for (size_t i0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i0 < n; i0 += (size_t)gridDim.x * blockDim.x) {
+        const size_t i = r * n + i0;
+        if (MODE == 0) {
+            for (int k = 0; k <= j; ++k) U[k][i] = cmac(R[k][i], c[0][0], U[k][i]);
+        } else if (MODE == 1) {
+            x[i] = cmac(x[i], c[1][0], U[0][i]);
+            for (int k = 0; k <= j; ++k) R[k][i] = cmac(R[k][i], c[0][0], U[k + 1][i]);
+        } else {
+            float2 xv = x[i], rv = R[0][i], uv = U[0][i];
+            xv = cmac(xv, c[0][0], rv);
+            for (int k = 1; k <= j; ++k) {
+                const float2 rk = R[k][i], uk = U[k][i];
+                xv = cmac(xv, c[0][k], rk);
+                rv = cmac(rv, c[1][k], rk);
+                uv = cmac(uv, c[2][k], uk);
+            }
+            x[i] = xv;
+            R[0][i] = rv;
+            U[0][i] = uv;
+        }
+    }
+}
+template <int K, bool GRAM>
+void batch_dot_launch(int k, const BatchVecs& a, const float2* b, size_t n, int nb, int gx, double2* part,
+                      cudaStream_t st) {
+    if constexpr (K > 1) {
+        if (k < K) return batch_dot_launch<K - 1, GRAM>(k, a, b, n, nb, gx, part, st);
+    }
+    (note_launch(), batch_dot_kernel<K, GRAM><<<dim3(gx, nb), kBT, 0, st>>>(a, b, n, part));
 }
 
 // ---- ragged batch: one Gram-Schmidt pass for every problem, one launch per step
@@ -389,6 +525,40 @@ cudaError_t launch_multi_dot_norm(int prec, int k, const void* const* a, const v
     for (int j = 0; j < k; ++j) pl.p[j] = a[j];
     if (prec == 0) multi_dot_launch<double2, kMaxDots - 1>(k, true, pl, (const double2*)b, n, partials, st);
     else multi_dot_launch<float2, kMaxDots - 1>(k, true, pl, (const float2*)b, n, partials, st);
+    return cudaGetLastError();
+}
+int batch_ctas(size_t n) {
+    const size_t c = (n + 4 * kBT - 1) / (4 * kBT);   // four entries per thread
+    return (int)(c < 1 ? 1 : c > (size_t)sm_count() ? sm_count() : c);
+}
+cudaError_t launch_batch_dot(int k, void* const* a, const void* b, size_t n, int nb, double2* part, cudaStream_t st) {
+    if (k < 1 || k > 5 || nb < 1 || nb > 16) return cudaErrorInvalidValue;
+    BatchVecs v = {};
+    for (int p = 0; p < k; ++p) v.v[p] = (float2*)a[p];
+    if (b) batch_dot_launch<5, false>(k, v, (const float2*)b, n, nb, batch_ctas(n), part, st);
+    else batch_dot_launch<5, true>(k, v, nullptr, n, nb, batch_ctas(n), part, st);
+    return cudaGetLastError();
+}
+cudaError_t launch_batch_update(int mode, int ell, void* const* R, void* const* U, void* x, const double2* coef,
+                                unsigned active, int j, size_t n, int nb, cudaStream_t st) {
+    if (ell < 1 || ell > 4 || j < 0 || j > ell || nb < 1 || nb > 16) return cudaErrorInvalidValue;
+    BatchVecs v = {};
+    for (int p = 0; p <= ell; ++p) {
+        v.v[p] = (float2*)R[p];
+        v.v[5 + p] = (float2*)U[p];
+    }
+    BatchCoefs c;
+    c.active = active;
+    for (int r = 0; r < nb; ++r)
+        for (int q = 0; q < 3; ++q)
+            for (int p = 0; p < kBatchCoef; ++p) {
+                const double2 t = coef[(r * 3 + q) * kBatchCoef + p];
+                c.c[r][q][p] = make_float2((float)t.x, (float)t.y);
+            }
+    const dim3 grid(batch_ctas(n), nb);
+    if (mode == 0) (note_launch(), batch_update_kernel<0><<<grid, kBT, 0, st>>>(v, (float2*)x, c, j, n));
+    else if (mode == 1) (note_launch(), batch_update_kernel<1><<<grid, kBT, 0, st>>>(v, (float2*)x, c, j, n));
+    else (note_launch(), batch_update_kernel<2><<<grid, kBT, 0, st>>>(v, (float2*)x, c, j, n));
     return cudaGetLastError();
 }
 cudaError_t launch_norm2(int prec, const void* a, size_t n, double* partials, cudaStream_t st) {

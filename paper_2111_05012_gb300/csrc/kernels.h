@@ -209,6 +209,16 @@ cudaError_t launch_coarse_op_export(int cprec, int Vc, int nc, const void* B, do
 cudaError_t launch_convert_flat(int prec_in, int prec_out, const void* in, void* out, size_t n, cudaStream_t s);
 
 // ---- BLAS-1 on flat complex arrays (prec 0 = double2, 1 = float2) ----
+// ---- batches of up to 16 FP32 complex vectors (right-hand side r of a field at r * n)
+int batch_ctas(size_t n);   // CTAs (partials) per reduced quantity
+// part[(r * k + p) * batch_ctas(n) + cta]: <a_p, b> for p < k <= 5; b null: all <a_p, a_q>, p <= q
+cudaError_t launch_batch_dot(int k, void* const* a, const void* b, size_t n, int nb, double2* part, cudaStream_t s);
+// BiCGStab(l) updates of the active right-hand sides (bit mask), coef[r][3][5]:
+// mode 0: U_i = R_i + c0 U_i, i <= j;  1: R_i += c0 U_{i+1}, i <= j, x += c1 U_0;
+// 2: x += sum c0_k R_k, R_0 += sum c1_k R_k, U_0 += sum c2_k U_k (k <= j, from the old R_0)
+cudaError_t launch_batch_update(int mode, int ell, void* const* R, void* const* U, void* x, const double2* coef,
+                                unsigned active, int j, size_t n, int nb, cudaStream_t s);
+
 // partial sums: per-CTA double2 partials written to `partials` (k dots of a[i] with b, grid CTAs each)
 int blas_grid();
 cudaError_t launch_multi_dot(int prec, int k, const void* const* a, const void* b, size_t n, double2* partials,
