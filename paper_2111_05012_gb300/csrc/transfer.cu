@@ -334,16 +334,7 @@ __global__ void prolong_ragged_kernel(const RaggedDev* __restrict__ d, const int
 // eps |w0| / |w| <= 2 eps otherwise (the DGKS test).  Either way the result is
 // the QR factor with a positive diagonal to rounding, the vectors that
 // projecting one vector after another gives.
-// FP64 runs at 1/64 of the FP32 rate, so the FP64 instructions are the time: fused multiply-adds
-// (48 per pair of vectors and site half), and FP32 values widened with integer instructions
-// instead of conversions on the FP64 pipe.  16^3 x 32, 24 vectors: 16.4 -> 11.8 ms.
-DEV double widen(float f) {
-    const unsigned u = __float_as_uint(f), e = (u >> 23) & 0xFFu;
-    if (e == 0 || e == 255) return (double)f;   // zero and subnormal values, infinities, NaN
-    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + (896u << 20))), (int)(u << 29));
-}
-DEV cx<double> widen(cx<float> a) { return {widen(a.re), widen(a.im)}; }
-DEV cx<double> widen(cx<double> a) { return a; }
+// FP64 vectors; FP32 vectors take orthonormalise_pairs_kernel.
 // chirality half chi of a fine field at one site (plain loads: written earlier in the launch)
 template <class PV> DEV void load_chirality(const void* base, int V, int s, int chi, cx<typename PV::T> v[6]);
 template <> DEV void load_chirality<P32>(const void* base, int V, int s, int chi, cx<float> v[6]) {
@@ -363,7 +354,6 @@ template <> DEV void load_chirality<P64>(const void* base, int V, int s, int chi
         v[k] = {t.x, t.y};
     }
 }
-template <class PV>
 __global__ void __launch_bounds__(512) orthonormalise_kernel(Geom g, Blocking bk, int nvec, void* vecs, int* err) {
     __shared__ double red[3 * 32];
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -372,16 +362,16 @@ __global__ void __launch_bounds__(512) orthonormalise_kernel(Geom g, Blocking bk
     const int Xi = blockIdx.x, chi = blockIdx.y;
     const int l = threadIdx.x, lane = l & 31, warp = l >> 5, nw = blockDim.x >> 5;
     const bool active = l < bk.Vb;
-    const size_t vb = spinor_bytes<PV>(g.V);
-    constexpr int G = PV::id == 0 ? 1 : 2;   // previous vectors in flight (more spill at the 128 registers of 512 threads)
+    const size_t vb = spinor_bytes<P64>(g.V);
+    constexpr int G = 1;   // previous vectors in flight (more spill at the 128 registers of 512 threads)
     int c[4], s = 0;
     if (active) s = block_site(g, bk, Xi, l, c);
     auto load_half = [&](int j, cx<double> (&q)[6]) {
         if (active) {
-            cx<typename PV::T> u[6];
-            load_chirality<PV>((const char*)vecs + j * vb, g.V, s, chi, u);
+            cx<double> u[6];
+            load_chirality<P64>((const char*)vecs + j * vb, g.V, s, chi, u);
 #pragma unroll
-            for (int k = 0; k < 6; ++k) q[k] = widen(u[k]);
+            for (int k = 0; k < 6; ++k) q[k] = u[k];
         } else {
 #pragma unroll
             for (int k = 0; k < 6; ++k) q[k] = czero<double>();
@@ -403,17 +393,17 @@ __global__ void __launch_bounds__(512) orthonormalise_kernel(Geom g, Blocking bk
             // G previous vectors at a time: their loads in flight together, and their sums taken over
             // the warp by transposed shuffles (10 FP64 additions for four sums instead of 20)
             for (int j0 = 0; j0 < i; j0 += G) {
-                cx<typename PV::T> u[G][6];
+                cx<double> u[G][6];
 #pragma unroll
                 for (int t = 0; t < G; ++t)
-                    if (active && j0 + t < i) load_chirality<PV>((const char*)vecs + (j0 + t) * vb, g.V, s, chi, u[t]);
+                    if (active && j0 + t < i) load_chirality<P64>((const char*)vecs + (j0 + t) * vb, g.V, s, chi, u[t]);
                 double q[2 * G];
 #pragma unroll
                 for (int t = 0; t < G; ++t) {
                     cx<double> d = czero<double>();
                     if (active && j0 + t < i) {
 #pragma unroll
-                        for (int k = 0; k < 6; ++k) cfmac(d, widen(u[t][k]), w[k]);
+                        for (int k = 0; k < 6; ++k) cfmac(d, u[t][k], w[k]);
                     }
                     q[2 * t] = d.re;
                     q[2 * t + 1] = d.im;
@@ -431,16 +421,16 @@ __global__ void __launch_bounds__(512) orthonormalise_kernel(Geom g, Blocking bk
             }
             __syncthreads();
             for (int j0 = 0; j0 < i; j0 += G) {
-                cx<typename PV::T> u[G][6];
+                cx<double> u[G][6];
 #pragma unroll
                 for (int t = 0; t < G; ++t)
-                    if (active && j0 + t < i) load_chirality<PV>((const char*)vecs + (j0 + t) * vb, g.V, s, chi, u[t]);
+                    if (active && j0 + t < i) load_chirality<P64>((const char*)vecs + (j0 + t) * vb, g.V, s, chi, u[t]);
 #pragma unroll
                 for (int t = 0; t < G; ++t) {
                     if (!active || j0 + t >= i) break;
                     const cx<double> cc = -coef[j0 + t];
 #pragma unroll
-                    for (int k = 0; k < 6; ++k) cfma(w[k], cc, widen(u[t][k]));
+                    for (int k = 0; k < 6; ++k) cfma(w[k], cc, u[t][k]);
                 }
             }
             __syncthreads();   // part / coef are rewritten by the next pass
@@ -448,8 +438,8 @@ __global__ void __launch_bounds__(512) orthonormalise_kernel(Geom g, Blocking bk
         double nn[1] = {0};
         for (int k = 0; k < 6; ++k) nn[0] += norm2(w[k]);
         block_sum<double, 1>(nn, red);
-        // rank test: |w| <= 1e-12 |w0| (FP64 storage), 1e-5 |w0| (FP32 storage)
-        const double rtol2 = PV::id == 0 ? 1e-24 : 1e-10;
+        // rank test: |w| <= 1e-12 |w0|
+        const double rtol2 = 1e-24;
         if (!(nn[0] > rtol2 * n0[0])) {
             if (threadIdx.x == 0) atomicExch(err, 1);
             nn[0] = 1.0;
@@ -457,9 +447,202 @@ __global__ void __launch_bounds__(512) orthonormalise_kernel(Geom g, Blocking bk
         double inv = 1.0 / sqrt(nn[0]);
         if (active) {
             // the other chirality half belongs to the CTA (Xi, 1 - chi): write ours only
-            cx<typename PV::T> hv[6];
-            for (int k = 0; k < 6; ++k) hv[k] = ccast<typename PV::T>(inv * w[k]);
-            SpinorIO<PV>::store_half((char*)vecs + i * vb, g.V, s, chi, hv);
+            cx<double> hv[6];
+            for (int k = 0; k < 6; ++k) hv[k] = ccast<double>(inv * w[k]);
+            SpinorIO<P64>::store_half((char*)vecs + i * vb, g.V, s, chi, hv);
+        }
+        __syncthreads();
+    }
+}
+
+// ---- FP32 vectors: the same Gram-Schmidt with the projected vector as float pairs (hi + lo, 48
+// bits) on the FP32 pipe.  The stored vectors are exact floats, so every product with one is an
+// exact product of floats plus a correction; the sums keep their rounding errors (two-sum), over
+// the warp as pairs, over the warps in FP64.  The result is rounded to FP32 as before: its error
+// against 64 bits is that rounding either way (8^4, 24 vectors: 2.55e-8, and 7.53e-7 for vectors that
+// differ by 1/30, with FP64 arithmetic as with pairs).  Eleven FP32 instructions stand for an
+// FP64 one of 1/64 the rate: 16^3 x 32, 24 vectors 11.8 -> 2.2 ms.
+DEV void pair_mac(dfloat& a, dfloat w, float q) {   // a += w q
+    const float p = __fmul_rn(w.hi, q);
+    float e = fmaf(w.hi, q, -p);
+    e = fmaf(w.lo, q, e);
+    const dfloat t = two_sum(a.hi, p);
+    a.hi = t.hi;
+    a.lo = __fadd_rn(a.lo, __fadd_rn(t.lo, e));
+}
+DEV void pair_square(dfloat& a, dfloat w) {   // a += w w
+    const float p = __fmul_rn(w.hi, w.hi);
+    float e = fmaf(w.hi, w.hi, -p);
+    e = fmaf(__fadd_rn(w.hi, w.hi), w.lo, e);
+    const dfloat t = two_sum(a.hi, p);
+    a.hi = t.hi;
+    a.lo = __fadd_rn(a.lo, __fadd_rn(t.lo, e));
+}
+DEV dfloat shfl_xor_pair(dfloat v, int off) {
+    return dfloat(__shfl_xor_sync(0xffffffffu, v.hi, off), __shfl_xor_sync(0xffffffffu, v.lo, off));
+}
+// sums of four pairs over the warp; lanes 8k .. 8k + 7 get the sum of value transposed_index<4>
+DEV dfloat transposed_pair_sum4(dfloat (&v)[4], int lane) {
+#pragma unroll
+    for (int h = 2, off = 16; h >= 1; h /= 2, off /= 2) {
+        const bool up = (lane & off) != 0;
+#pragma unroll
+        for (int k = 0; k < h; ++k) {
+            const dfloat keep = up ? v[k + h] : v[k], give = up ? v[k] : v[k + h];
+            v[k] = keep + shfl_xor_pair(give, off);
+        }
+    }
+    dfloat r = v[0];
+#pragma unroll
+    for (int off = 4; off >= 1; off /= 2) r = r + shfl_xor_pair(r, off);
+    return r;
+}
+// |w|^2 of the block (every thread gets it); one pair per warp through red, contains barriers
+DEV double pair_norm(const dfloat (&wr)[6], const dfloat (&wi)[6], double* red) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    dfloat n;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        pair_square(n, wr[k]);
+        pair_square(n, wi[k]);
+    }
+    n = quick_two_sum(n.hi, n.lo);
+#pragma unroll
+    for (int off = 16; off >= 1; off /= 2) n = n + shfl_xor_pair(n, off);
+    if (lane == 0) red[warp] = to_double(n);
+    __syncthreads();
+    double t = 0;
+    for (int w = 0; w < nw; ++w) t += red[w];
+    __syncthreads();
+    return t;
+}
+__global__ void __launch_bounds__(512) orthonormalise_pairs_kernel(Geom g, Blocking bk, int nvec, void* vecs, int* err) {
+    __shared__ double red[32];
+    __shared__ float redm[32];
+    __shared__ float2 s_inv;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    float2* part = reinterpret_cast<float2*>(smem_raw);                    // [nwarps][nvec][re, im] pairs
+    float4* coef = reinterpret_cast<float4*>(part + (size_t)nw * nvec * 2);   // [nvec]: re.hi, re.lo, im.hi, im.lo
+    const int Xi = blockIdx.x, chi = blockIdx.y;
+    const int l = threadIdx.x;
+    const bool active = l < bk.Vb;
+    const size_t vb = spinor_bytes<P32>(g.V);
+    int c[4], s = 0;
+    if (active) s = block_site(g, bk, Xi, l, c);
+    for (int i = 0; i < nvec; ++i) {
+        // w scaled by the power of two that brings its largest component on this domain to [1, 2)
+        // (exact, and the result does not depend on it): squares of any FP32 values stay in range
+        dfloat wr[6], wi[6];
+        cx<float> u0[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) u0[k] = czero<float>();
+        if (active) load_chirality<P32>((const char*)vecs + i * vb, g.V, s, chi, u0);
+        float m = 0.f;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) m = fmaxf(m, fmaxf(fabsf(u0[k].re), fabsf(u0[k].im)));
+#pragma unroll
+        for (int off = 16; off >= 1; off /= 2) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+        if (lane == 0) redm[warp] = m;
+        __syncthreads();
+        for (int w = 0; w < nw; ++w) m = fmaxf(m, redm[w]);
+        const int e = (int)(__float_as_uint(m) >> 23);   // biased exponent; 0: zero or subnormal
+        const float sc = m > 0.f && e < 255 ? __uint_as_float((unsigned)min(253, max(1, 254 - e)) << 23) : 1.f;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            wr[k] = dfloat(sc * u0[k].re);
+            wi[k] = dfloat(sc * u0[k].im);
+        }
+        const double n0 = pair_norm(wr, wi, red);   // its barriers keep redm's readers from the next writers
+        double nn = n0;
+        for (int pass = 0; pass < 2 && i > 0; ++pass) {
+            // a second projection only after a large cancellation
+            if (pass == 1 && nn > 0.25 * n0) break;
+            for (int j0 = 0; j0 < i; j0 += 2) {
+                cx<float> u[2][6];
+#pragma unroll
+                for (int t = 0; t < 2; ++t)
+                    if (active && j0 + t < i) load_chirality<P32>((const char*)vecs + (j0 + t) * vb, g.V, s, chi, u[t]);
+                dfloat q[4];
+#pragma unroll
+                for (int t = 0; t < 2; ++t) {
+                    dfloat re, im;   // <v_j, w>
+                    if (active && j0 + t < i) {
+#pragma unroll
+                        for (int k = 0; k < 6; ++k) {
+                            pair_mac(re, wr[k], u[t][k].re);
+                            pair_mac(re, wi[k], u[t][k].im);
+                            pair_mac(im, wi[k], u[t][k].re);
+                            pair_mac(im, wr[k], -u[t][k].im);
+                        }
+                    }
+                    q[2 * t] = quick_two_sum(re.hi, re.lo);
+                    q[2 * t + 1] = quick_two_sum(im.hi, im.lo);
+                }
+                const dfloat tot = transposed_pair_sum4(q, lane);
+                const int v = transposed_index<4>(lane);
+                if ((lane & 7) == 0 && j0 + (v >> 1) < i)
+                    part[((size_t)warp * nvec + j0 + (v >> 1)) * 2 + (v & 1)] = make_float2(tot.hi, tot.lo);
+            }
+            __syncthreads();
+            for (int j = l; j < i; j += blockDim.x) {
+                double re = 0, im = 0;
+                for (int w = 0; w < nw; ++w) {
+                    const float2 a = part[((size_t)w * nvec + j) * 2], b = part[((size_t)w * nvec + j) * 2 + 1];
+                    re += (double)a.x + (double)a.y;
+                    im += (double)b.x + (double)b.y;
+                }
+                const dfloat r = split_double(re), m = split_double(im);
+                coef[j] = make_float4(r.hi, r.lo, m.hi, m.lo);
+            }
+            __syncthreads();
+            for (int j0 = 0; j0 < i; j0 += 2) {
+                cx<float> u[2][6];
+#pragma unroll
+                for (int t = 0; t < 2; ++t)
+                    if (active && j0 + t < i) load_chirality<P32>((const char*)vecs + (j0 + t) * vb, g.V, s, chi, u[t]);
+#pragma unroll
+                for (int t = 0; t < 2; ++t) {
+                    if (!active || j0 + t >= i) break;
+                    const float4 cc = coef[j0 + t];   // w -= c v_j
+                    const dfloat nr(-cc.x, -cc.y), ni(-cc.z, -cc.w), pi(cc.z, cc.w);
+#pragma unroll
+                    for (int k = 0; k < 6; ++k) {
+                        pair_mac(wr[k], nr, u[t][k].re);
+                        pair_mac(wr[k], pi, u[t][k].im);
+                        pair_mac(wi[k], nr, u[t][k].im);
+                        pair_mac(wi[k], ni, u[t][k].re);
+                    }
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {   // the low parts gathered corrections: back to proper pairs
+                wr[k] = two_sum(wr[k].hi, wr[k].lo);
+                wi[k] = two_sum(wi[k].hi, wi[k].lo);
+            }
+            nn = pair_norm(wr, wi, red);   // also keeps part / coef readers apart from the next pass
+        }
+        // rank test: |w| <= 1e-5 |w0| (FP32 storage)
+        if (threadIdx.x == 0) {
+            double t = nn;
+            if (!(t > 1e-10 * n0)) {
+                atomicExch(err, 1);
+                t = 1.0;
+            }
+            const dfloat v = split_double(1.0 / sqrt(t));
+            s_inv = make_float2(v.hi, v.lo);
+        }
+        __syncthreads();
+        if (active) {
+            // the other chirality half belongs to the CTA (Xi, 1 - chi): write ours only
+            const dfloat inv(s_inv.x, s_inv.y);
+            cx<float> hv[6];
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                const dfloat a = inv * wr[k], b = inv * wi[k];
+                hv[k] = {a.hi, b.hi};
+            }
+            SpinorIO<P32>::store_half((char*)vecs + i * vb, g.V, s, chi, hv);
         }
         __syncthreads();
     }
@@ -728,8 +911,8 @@ cudaError_t launch_orthonormalise_fine(int vprec, const GeomH& gh, const BlockH&
     dim3 grid(bk.Vc, 2);
     int th = threads_for(bk);
     const size_t smem = ((size_t)(th / 32) + 1) * nvec * sizeof(cx<double>);
-    if (vprec == 0) (note_launch(), orthonormalise_kernel<P64><<<grid, th, smem, st>>>(g, bk, nvec, vecs, err));
-    else (note_launch(), orthonormalise_kernel<P32><<<grid, th, smem, st>>>(g, bk, nvec, vecs, err));
+    if (vprec == 0) (note_launch(), orthonormalise_kernel<<<grid, th, smem, st>>>(g, bk, nvec, vecs, err));
+    else (note_launch(), orthonormalise_pairs_kernel<<<grid, th, smem, st>>>(g, bk, nvec, vecs, err));
     return cudaGetLastError();
 }
 cudaError_t launch_galerkin_fine(int vprec, int cprec, const GeomH& gh, const BlockH& bh, int nvec, const void* vecs,
