@@ -124,15 +124,17 @@ struct RawHop {
         v.load(f, g.V, h.n);
         if (d > 0) l.load(U, g.V, (d - 1) & 3, h.link);
     }
-    // (T_d f)(s)
-    DEV void get(int d, cx<float> out[12]) const {
+    // (T_d f)(s), times the power of two sc
+    DEV void get(int d, cx<float> out[12], float sc = 1.f) const {
         if (d == 0) {
             v.get(out);
+#pragma unroll
+            for (int k = 0; k < 12; ++k) out[k] = sc * out[k];
             return;
         }
         cx<float> f[12], u[3][3];
         v.get(f);
-        l.get(ph, u);
+        l.get(sc * ph, u);
         colour_mul(u, d <= 4 ? 1 : -1, f, out);
     }
 };
@@ -162,32 +164,56 @@ DEV void add_square(dfloat& acc, float v) {
     acc.lo = __fadd_rn(acc.lo, __fadd_rn(t.lo, e));
 }
 
+// A thread's sum of squares of any FP32 values: a site whose largest component lies outside
+// [2^-50, 2^50] is scaled by a power of two first (FP32 squares would be lost or overflow) and its
+// sum goes to a double; the others' pairs add up as pairs
+struct SquareSum {
+    dfloat p;
+    double d = 0;
+    // the 24 components of a site, v(k)
+    template <class F> DEV void add(F&& v) {
+        float m = 0.f, q = 0.f;
+#pragma unroll
+        for (int k = 0; k < 24; ++k) m = fmaxf(m, fabsf(v(k)));
+        const float sc = m < 0x1p-50f ? 0x1p100f : m > 0x1p50f ? 0x1p-100f : 1.f;
+        dfloat t;
+#pragma unroll
+        for (int k = 0; k < 24; ++k) {
+            const float x = sc * v(k);
+            add_square(t, x);
+            q = fmaf(x, x, q);
+        }
+        if (!(q <= 0x1.fffffep127f)) d += q;   // infinite or NaN: the pair would turn both into NaN
+        else if (sc == 1.f) p = p + quick_two_sum(t.hi, t.lo);
+        else d += to_double(t) * (sc > 1.f ? 0x1p-200 : 0x1p200);
+    }
+    DEV double get() const { return to_double(p) + d; }
+};
+
 // The last layer of a training pass: y is replaced by y - e for the canonical target e, and
 // part[cta] receives the CTA's shares of |y - e|^2 and |e|^2
 struct LossArgs {
     const float4* e;   // canonical, 6 float4 per site; null outside training
     double2* part;
 };
-DEV void loss_site(const LossArgs& l, int s, cx<float> acc[12], dfloat& d2, dfloat& e2) {
+DEV void loss_site(const LossArgs& l, int s, cx<float> acc[12], SquareSum& d2, SquareSum& e2) {
+    float e[24];
 #pragma unroll
     for (int q = 0; q < 6; ++q) {
-        const float4 e = __ldg(l.e + (size_t)s * 6 + q);
-        acc[2 * q] = acc[2 * q] - cx<float>{e.x, e.y};
-        acc[2 * q + 1] = acc[2 * q + 1] - cx<float>{e.z, e.w};
-        add_square(e2, e.x);
-        add_square(e2, e.y);
-        add_square(e2, e.z);
-        add_square(e2, e.w);
+        const float4 t = __ldg(l.e + (size_t)s * 6 + q);
+        acc[2 * q] = acc[2 * q] - cx<float>{t.x, t.y};
+        acc[2 * q + 1] = acc[2 * q + 1] - cx<float>{t.z, t.w};
+        e[4 * q] = t.x;
+        e[4 * q + 1] = t.y;
+        e[4 * q + 2] = t.z;
+        e[4 * q + 3] = t.w;
     }
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-        add_square(d2, acc[k].re);
-        add_square(d2, acc[k].im);
-    }
+    e2.add([&](int k) { return e[k]; });
+    d2.add([&](int k) { return k & 1 ? acc[k >> 1].im : acc[k >> 1].re; });
 }
-DEV void loss_block(const LossArgs& l, dfloat d2, dfloat e2) {
+DEV void loss_block(const LossArgs& l, const SquareSum& d2, const SquareSum& e2) {
     __shared__ double red[2 * 32];
-    double v[2] = {to_double(d2), to_double(e2)};
+    double v[2] = {d2.get(), e2.get()};
     block_sum<double, 2>(v, red);
     if (threadIdx.x == 0) l.part[blockIdx.x] = make_double2(v[0], v[1]);
 }
@@ -199,7 +225,7 @@ DEV void loss_block(const LossArgs& l, dfloat d2, dfloat e2) {
 // Bound by the FP32 pipe (16 cin cout 9 complex spin entries x 3 colours per site, the
 // transports 8 x 36 complex products per transported channel).  128 threads, so that 160
 // registers still leave three CTAs per SM; the loop over the directions stays rolled to keep the
-// body in the instruction cache.  24^3 x 48: 1 -> 4 channels 331 -> 258 us, 4 -> 1 501 -> 321 us (loss included).
+// body in the instruction cache.  24^3 x 48: 1 -> 4 channels 331 -> 258 us, 4 -> 1 501 -> 332 us (loss included).
 constexpr int kFT = 128;
 DEV void load_weights(cx<float>* w, const __nv_bfloat16* __restrict__ W, int nw) {
     for (int i = threadIdx.x; i < nw; i += blockDim.x)
@@ -213,7 +239,7 @@ __global__ void __launch_bounds__(kFT, COUT >= 3 ? 3 : 4) ptconv_up_kernel(Geom 
     __shared__ __align__(16) cx<float> w[COUT * COUT * 9 * 16];   // cin <= COUT
     load_weights(w, W, COUT * cin * 9 * 16);
     const size_t fb = spinor_bytes<P32>(g.V);
-    dfloat d2, e2;
+    SquareSum d2, e2;
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < g.V; s += gridDim.x * blockDim.x) {
         int c[4];
         site_coords(g, s, c);
@@ -250,7 +276,7 @@ __global__ void __launch_bounds__(kFT, 3) ptconv_down_kernel(Geom g, int cout, c
     __shared__ __align__(16) cx<float> w[CIN * (CIN > 1 ? CIN - 1 : 1) * 9 * 16];   // cout < CIN
     load_weights(w, W, cout * CIN * 9 * 16);
     const size_t fb = spinor_bytes<P32>(g.V);
-    dfloat d2, e2;
+    SquareSum d2, e2;
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < g.V; s += gridDim.x * blockDim.x) {
         int c[4];
         site_coords(g, s, c);
@@ -307,13 +333,21 @@ __global__ void __launch_bounds__(kFT, 3) ptconv_down_kernel(Geom g, int cout, c
 // the products.  blockIdx.y: the transported channel.
 // Every kFlush sites per lane the sums move on, over the warp, into float pairs (48 bits), so
 // the plain FP32 accumulation is no longer than a few sites.  24^3 x 48, four static channels:
-// 1 -> 4 layer 757 -> 472 us, 4 -> 1 layer 1140 -> 451 us; bound by the FP32 pipe and by latency
+// 1 -> 4 layer 757 -> 479 us, 4 -> 1 layer 1140 -> 459 us; bound by the FP32 pipe and by latency
 // at eight warps per SM.
 // part[(blockIdx.y * 9 + d) * max(gridDim.x - n0, n0) + cta][NS * 16]
 constexpr int kWT = 256, kFlush = 8;
+// Power of two on the transported side of a training pair of very small or large targets: in and
+// y - e scale alike, and their FP32 products would leave the range long before the fields do
+DEV float grad_scale(const double2* __restrict__ norm) {
+    if (!norm || !(norm->y > 0) || (norm->y >= 0x1p-60 && norm->y <= 0x1p80)) return 1.f;
+    return (float)exp2((double)max(-120, min(120, -ilogb(norm->y) / 2)));
+}
 template <int NS, bool ADJ>
 __global__ void __launch_bounds__(kWT, 1) ptconv_wgrad_kernel(Geom g, const void* __restrict__ U, const void* moved,
-                                                              const void* fixed, int n0, double2* part) {
+                                                              const void* fixed, int n0, double2* part,
+                                                              const double2* __restrict__ norm) {
+    const float psc = grad_scale(norm);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool self = (int)blockIdx.x < n0;
     const int d = self ? 0 : warp + 1;
@@ -357,7 +391,7 @@ __global__ void __launch_bounds__(kWT, 1) ptconv_wgrad_kernel(Geom g, const void
             RawSpinor r;
             r.load(fixed, g.V, s);
             cx<float> phi[12];
-            h.get(td, phi);
+            h.get(td, phi, psc);
             fetch(s + step);
 #pragma unroll
             for (int a = 0; a < NS; ++a) {
@@ -427,7 +461,7 @@ __global__ void __launch_bounds__(256) ptconv_wsum_kernel(int cin, int ns, int n
     if (lane == 0) {
         const int a = adj ? m : q / 16, b = adj ? q / 16 : m;
         double2& o = G[(((size_t)a * cin + b) * 9 + d) * 16 + q % 16];
-        const double sc = norm ? 1.0 / norm->y : 1.0;
+        const double sc = (norm ? 1.0 / norm->y : 1.0) / grad_scale(norm);
         o = make_double2((add ? o.x : 0.0) + sc * re, (add ? o.y : 0.0) + sc * im);
     }
 }
@@ -495,7 +529,7 @@ cudaError_t launch_ptconv_wgrad(const GeomH& gh, int cin, int cout, const void* 
     const int need = (g.V + 31) / 32, n8 = std::min(need, std::max(1, sms() - sms() / 10));
     const int n0 = std::min((need + 7) / 8, std::max(1, sms() / 10));
     const dim3 grid(n0 + n8, nm);
-#define WG(N, A) (note_launch(), ptconv_wgrad_kernel<N, A><<<grid, kWT, 0, st>>>(g, U32, A ? gout : in, A ? in : gout, n0, part))
+#define WG(N, A) (note_launch(), ptconv_wgrad_kernel<N, A><<<grid, kWT, 0, st>>>(g, U32, A ? gout : in, A ? in : gout, n0, part, norm))
     switch (ns) {
         case 1: WG(1, false); break;
         case 2: if (adj) WG(2, true); else WG(2, false); break;
