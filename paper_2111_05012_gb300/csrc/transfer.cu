@@ -660,8 +660,10 @@ __global__ void __launch_bounds__(512) orthonormalise_pairs_kernel(Geom g, Block
 // shared memory and the CTA's threads split into groups over the same face
 // sites, each group projecting on its share of the test vectors: the vectors
 // are read from L2 for 3 blocks' worth of sites per column pair instead of
-// 6.5 (every warp has sites of most faces).  16^3 x 32, 24 vectors: 11.0 ->
-// 6.9 ms; bound by the L2 (every column pair reads the block's vectors).
+// 6.5 (every warp has sites of most faces).  The column pairs of a block are
+// neighbours in the grid, so that 23 of 24 find its vectors in L2 (blocks first,
+// the 302 MB of vectors came from DRAM for every pair, 5.3 TB/s of it).  16^3 x
+// 32, 24 vectors: 11.0 -> 3.7 ms; bound by the latency of L2 at 16 warps per SM.
 template <class PV, typename TC>
 __global__ void __launch_bounds__(PV::id == 0 ? 256 : 512) galerkin_kernel(Geom g, Blocking bk, int nvec, const void* __restrict__ vecs,
                                 const void* __restrict__ U, const void* __restrict__ C, typename PV::T kappa,
@@ -674,7 +676,8 @@ __global__ void __launch_bounds__(PV::id == 0 ? 256 : 512) galerkin_kernel(Geom 
     T* partf = reinterpret_cast<T*>(smem_raw);   // [nwarps][2 columns][nc] complex
     cx<T>* part = reinterpret_cast<cx<T>*>(smem_raw);
     cx<T>* tsh = part + (size_t)nw * 2 * nc;     // [2 columns][12][face sites, padded]
-    const int Xi = blockIdx.x, Ja = 2 * blockIdx.y, Jb = Ja + 1;
+    // the pairs of one block follow each other: they read the block's vectors from L2
+    const int Xi = blockIdx.x / nvec, Ja = 2 * (blockIdx.x % nvec), Jb = Ja + 1;
     const bool hasB = Jb < nc;
     const int ta = Ja / nvec, ja = Ja % nvec, tb = hasB ? Jb / nvec : 0, jb = hasB ? Jb % nvec : 0;
     const size_t vb = spinor_bytes<PV>(g.V);
@@ -685,7 +688,10 @@ __global__ void __launch_bounds__(PV::id == 0 ? 256 : 512) galerkin_kernel(Geom 
     auto load_proj = [&](const char* v, int t, int site, cx<T> out[12]) {
         SpinorIO<PV>::load(v, g.V, site, out);
 #pragma unroll
-        for (int k = 0; k < 6; ++k) out[6 * (1 - t) + k] = czero<T>();
+        for (int k = 0; k < 6; ++k) {   // selects, so that the spinor stays in registers
+            if (t != 0) out[k] = czero<T>();
+            else out[6 + k] = czero<T>();
+        }
     };
     // acc_a += coeff (1 - dir gamma_mu) W P_ta v_ja(n), acc_b likewise (one link load)
     auto hop2 = [&](int n, int linksite, int mu, int dir, T coeff, cx<T> (&acc_a)[12], cx<T> (&acc_b)[12]) {
@@ -729,6 +735,7 @@ __global__ void __launch_bounds__(PV::id == 0 ? 256 : 512) galerkin_kernel(Geom 
                     load_proj(vbp, tb, s, psi);
                     clover_apply<PV>(C, g.V, s, psi, Tb);
                 }
+#pragma unroll
                 for (int m = 0; m < 4; ++m) {
                     const int lc = c[m] % bk.b[m];
                     if (lc != bk.b[m] - 1) {
@@ -741,8 +748,17 @@ __global__ void __launch_bounds__(PV::id == 0 ? 256 : 512) galerkin_kernel(Geom 
                     }
                 }
             } else {
-                int n = neighbour(g, s, c, mu, dir, ph);
-                hop2(n, dir > 0 ? s : n, mu, dir, -kappa * T(ph), Ta, Tb);
+                // the direction is uniform; unrolled so that the spinors are indexed by constants
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    if (d == 1 + m) {
+                        const int n = neighbour(g, s, c, m, +1, ph);
+                        hop2(n, s, m, +1, -kappa * T(ph), Ta, Tb);
+                    } else if (d == 5 + m) {
+                        const int n = neighbour(g, s, c, m, -1, ph);
+                        hop2(n, n, m, -1, -kappa * T(ph), Ta, Tb);
+                    }
+                }
             }
             if (ngrp > 1) {
 #pragma unroll
@@ -920,7 +936,7 @@ cudaError_t launch_galerkin_fine(int vprec, int cprec, const GeomH& gh, const Bl
     Geom g = make_geom(gh);
     Blocking bk = make_blocking(gh, bh);
     int th = threads_for(bk);
-    dim3 grid(bk.Vc, nvec);   // pairs of columns
+    const unsigned grid = (unsigned)bk.Vc * nvec;   // block, pair of columns (nvec pairs: 2 nvec columns)
     // T of the largest face that leaves room for a second group of threads
     size_t face = 0;
     for (int mu = 0; mu < 4; ++mu) {
