@@ -154,11 +154,9 @@ def dist_info():
     return rank, world, local
 
 
-SAP_DRAM_BYTES_PER_SITE_RHS = 1378.0
-SAP_KERNEL_NAMES = {0: "sap_half_kernel<P32,256> (fused SAP half sweep)",
-                    1: "sap_half_staged_kernel<P32> (fused SAP half sweep, operator staged in shared memory)",
-                    2: "sap_half_kernel<P32,256,2> (fused SAP half sweep, two right-hand sides per CTA)",
-                    3: "sap_half_staged_kernel<P32,P16> (fused SAP half sweep, FP16 operator staged in shared memory)"}
+SAP_DRAM_BYTES_PER_SITE_RHS = 776.0
+SAP_KERNEL_NAMES = {3: "sap_half_staged_kernel<P32,P16> (fused SAP half sweep, FP16 operator staged in shared memory)"}
+SAP_KERNEL = "sap_pairs_kernel<P32> (fused SAP half sweep, packed FP32 pairs)"
 
 
 def make_params(capi, prec_smoother, coarse="f32", outer="fgmres", sap_variant=-1, setup=None, vec="f32", w=None):
@@ -433,12 +431,12 @@ def run_headline(args):
     flop_step = flop_site * (V / 2) * 2 * p.sap_iters * cycles * ns
     sap_tflops = flop_step / (smooth_ms * 1e-3) / 1e12
     # DRAM traffic of one launch (one colour, the batch's right-hand sides), scaled from an ncu
-    # capture of sap_half_kernel<P32,256,1> on 24^3x48 with 12 right-hand sides per launch
-    # (dram__bytes_read.sum + dram__bytes_write.sum = 2.372 + 0.371 GB over 165,888 active sites x
-    # 12 right-hand sides = 1378 B per active site and right-hand side); variant 0 only
+    # capture of sap_pairs_kernel<P32> on 24^3x48 with 4 right-hand sides per launch
+    # (dram__bytes_read.sum + dram__bytes_write.sum = 0.916 + 0.114 GB over 331,776 active sites x
+    # 4 right-hand sides = 776 B per active site and right-hand side); not for variant 3
     width = max(int(i.get("batch_width", 0)) for i in infos) or 1
     sap_traffic = (SAP_DRAM_BYTES_PER_SITE_RHS * (V / 2) * width
-                   if (args.sap_variant == 0 and not p.sap_eo) else None)
+                   if (args.sap_variant != 3 and not p.sap_eo) else None)
     hbm, kind = _peaks()
     # the other kernels the metric names, timed alone on this workload's fields
     kern = {}
@@ -478,7 +476,7 @@ def run_headline(args):
         "warmup": args.warmup, "ms_per_step": ms_step, "higher_is_better": False, "scaling": "weak",
         "vs_baseline": None, "dtype": "f32+f16+f64", "data": "synthetic", "config": config,
         "roofline": {"kernel": ("sap_half_eo_kernel<P32> (fused SAP half sweep, even-odd domain solves)"
-                               if p.sap_eo else SAP_KERNEL_NAMES.get(args.sap_variant, "sap_half (autotuned)")),
+                               if p.sap_eo else SAP_KERNEL_NAMES.get(args.sap_variant, SAP_KERNEL)),
                      "bound": "alu",
                      "achieved": sap_tflops, "peak": peak, "unit": "TFLOP/s", "frac": sap_tflops / peak,
                      "traffic": sap_traffic, "rhs_per_launch": width,
@@ -1087,13 +1085,13 @@ def run_solve16(args):
                                 ("ms_coarse", "ms_smoother", "ms_restrict_prolong", "ms_other", "ms_products",
                                  "ms_orthogonalisation", "ms_true_residual")},
                    "coarse_cycles": float(np.mean([i["coarse_cycles"] for i in infos]))},
-        # traffic: the per-site DRAM count of the current kernel's capture (24^3x48, 12 right-hand
-        # sides per launch) scaled to this workload's launches (one right-hand side); variant 0 only
-        "roofline": {"kernel": SAP_KERNEL_NAMES.get(args.sap_variant, "sap_half (autotuned)"),
+        # traffic: the per-site DRAM count of the kernel's capture (24^3x48, 4 right-hand sides per
+        # launch) scaled to this workload's launches (one right-hand side); not for variant 3
+        "roofline": {"kernel": SAP_KERNEL_NAMES.get(args.sap_variant, SAP_KERNEL),
                      "bound": "alu", "achieved": achieved, "peak": peak,
                      "unit": "TFLOP/s", "frac": achieved / peak,
                      "traffic": (SAP_DRAM_BYTES_PER_SITE_RHS * V / 2
-                                 if (args.sap_variant == 0 and args.prec == "f32") else None),
+                                 if (args.sap_variant != 3 and args.prec == "f32") else None),
                      "peak_kind": f"FP32 FMA from unit counts: {sms} SMs x 128 lanes x 2 flop x {mhz:.0f} MHz",
                      "avg_launch_us": sap_launch_us, "flop_per_launch": flop_launch,
                      "hbm_peak_gbs": hbm_peak, "hbm_peak_kind": peak_kind},
@@ -1147,8 +1145,8 @@ def main():
     ap.add_argument("--fused-only", action="store_true",
                     help="ragged workload: time the fused batch only (no stream-pool or one-by-one comparison)")
     ap.add_argument("--sap-variant", type=int, default=0, choices=[-1, 0, 1, 2, 3],
-                    help="SAP kernel: 0 operator through L1/L2 (default), 1 staged in shared memory, "
-                         "2 two right-hand sides of a batch per CTA, -1 autotune")
+                    help="SAP kernel: 3 FP16 operator staged in shared memory, the others packed FP32 pairs "
+                         "with the operator through L1/L2 (default)")
     ap.add_argument("--n-init", type=int, default=None, help="setup (0-a) SAP applications (default: library's)")
     ap.add_argument("--n-adapt", type=int, default=None, help="setup (0-b) adaptive passes (default: library's)")
     ap.add_argument("--coarse-tol", type=float, default=None, help="coarsest solve tolerance (default: library's)")
