@@ -943,16 +943,21 @@ cudaError_t launch_galerkin_fine(int vprec, int cprec, const GeomH& gh, const Bl
         const size_t nfp = (bk.Vb / bk.b[mu] + 31) / 32 * 32;
         if (th >= (int)(2 * nfp) && 24 * nfp > face) face = 24 * nfp;
     }
-    if (vprec == 0) {
-        const size_t smem = ((size_t)(th / 32) * 2 * 2 * nvec + face) * sizeof(cx<double>);
-        if (cprec == 0) (note_launch(), galerkin_kernel<P64, double><<<grid, th, smem, st>>>(g, bk, nvec, vecs, U, C, kappa, B));
-        else (note_launch(), galerkin_kernel<P64, float><<<grid, th, smem, st>>>(g, bk, nvec, vecs, U, C, kappa, B));
-    } else {
-        const size_t smem = ((size_t)(th / 32) * 2 * 2 * nvec + face) * sizeof(cx<float>);
-        if (cprec == 0) (note_launch(), galerkin_kernel<P32, double><<<grid, th, smem, st>>>(g, bk, nvec, vecs, U, C, (float)kappa, B));
-        else (note_launch(), galerkin_kernel<P32, float><<<grid, th, smem, st>>>(g, bk, nvec, vecs, U, C, (float)kappa, B));
-    }
-    return cudaGetLastError();
+    // Partial sums and face tile: past the 48 KB that a launch gets unasked for blocks with an extent
+    // of two (24 x 256 face sites of FP32 are 48 KB by themselves) and for FP64 blocks of many vectors;
+    // 80 KB at 64 vectors on 512 (FP32) or 256 (FP64) threads.  The limit is always set to that bound:
+    // a launch from another thread never finds it lowered to a smaller block's need.
+    constexpr int kSmemBound = 80 * 1024;
+    const size_t smem = ((size_t)(th / 32) * 2 * 2 * nvec + face) * (vprec == 0 ? sizeof(cx<double>) : sizeof(cx<float>));
+    auto launch = [&](auto kernel, auto kap) -> cudaError_t {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBound);
+        if (e != cudaSuccess) return e;
+        (note_launch(), kernel<<<grid, th, smem, st>>>(g, bk, nvec, vecs, U, C, kap, B));
+        return cudaGetLastError();
+    };
+    if (vprec == 0) return cprec == 0 ? launch(galerkin_kernel<P64, double>, kappa) : launch(galerkin_kernel<P64, float>, kappa);
+    return cprec == 0 ? launch(galerkin_kernel<P32, double>, (float)kappa)
+                      : launch(galerkin_kernel<P32, float>, (float)kappa);
 }
 
 // ---------------------------------------------------------------- ragged batches
