@@ -2863,6 +2863,15 @@ static amg_status transfer_common(amg_hierarchy* h, int coarsening, int nrhs, am
     return AMG_OK;
 }
 
+// the FP32 kernels on the caller's vectors need them apart from each other: overlapping ones go
+// through a scratch field, which holds one side while the other is read or written
+static bool transfer_apart(amg_hierarchy* h, const void* fine, const void* coarse, int nrhs) {
+    const size_t fb = (size_t)fine_geom(h).V * 24 * sizeof(float) * nrhs;
+    const size_t cb = coarse_n(h->lev[1]) * 2 * sizeof(float) * nrhs;
+    const char *f = (const char*)fine, *c = (const char*)coarse;
+    return f + fb <= c || c + cb <= f;
+}
+
 // Eqs. 5-6 from coarse level l >= 1: canonical = internal coarse layout; vectors
 // converted around the kernel when the caller's precision is not the level's
 static amg_status coarse_transfer(amg_hierarchy* h, int l, bool restrict_dir, const void* in, void* out, int nrhs,
@@ -2898,7 +2907,7 @@ amg_status amg_restrict(amg_hierarchy* h, int coarsening, const void* fine, void
     const GeomH& g = fine_geom(h);
     cudaStream_t st = (cudaStream_t)s;
     int cprec = prec == AMG_F64 ? 0 : 1;
-    if (prec == AMG_F32 && transfer_canon_supported(h->rp, cprec, fine)) {
+    if (prec == AMG_F32 && transfer_canon_supported(h->rp, cprec, fine) && transfer_apart(h, fine, coarse, nrhs)) {
         // the caller's vectors as they are: no copy to the internal layout, no scratch
         CK(launch_restrict_canon(h->rp, g, h->blk[0], h->p.nvec[0], rp_vecs(h), fine, coarse, nrhs, st));
         return AMG_OK;
@@ -2918,7 +2927,7 @@ amg_status amg_prolong(amg_hierarchy* h, int coarsening, const void* coarse, voi
     const GeomH& g = fine_geom(h);
     cudaStream_t st = (cudaStream_t)s;
     int cprec = prec == AMG_F64 ? 0 : 1;
-    if (prec == AMG_F32 && transfer_canon_supported(h->rp, cprec, fine)) {
+    if (prec == AMG_F32 && transfer_canon_supported(h->rp, cprec, fine) && transfer_apart(h, fine, coarse, nrhs)) {
         CK(launch_prolong_canon(h->rp, g, h->blk[0], h->p.nvec[0], rp_vecs(h), coarse, fine, nrhs, st));
         return AMG_OK;
     }
