@@ -364,7 +364,9 @@ amg_status amg_coarse_time(amg_hierarchy* h, int level, const void* in, int nrhs
 
 /* Eq. 5: coarse(I) = <I|fine> from level `coarsening` to coarsening+1.
  * fine is canonical at that level (a fine field for coarsening 0, a coarse
- * vector [site][Nc] for coarsening >= 1); element type from prec as above. */
+ * vector [site][Nc] for coarsening >= 1); element type from prec as above.
+ * amg_restrict and amg_prolong wait for the stream: the result is complete on
+ * return, in every precision and for vectors of any alignment. */
 amg_status amg_restrict(amg_hierarchy* h, int coarsening, const void* fine, void* coarse, int nrhs,
                         amg_prec prec, amg_stream s);
 

@@ -2910,6 +2910,7 @@ amg_status amg_restrict(amg_hierarchy* h, int coarsening, const void* fine, void
     if (prec == AMG_F32 && transfer_canon_supported(h->rp, cprec, fine) && transfer_apart(h, fine, coarse, nrhs)) {
         // the caller's vectors as they are: no copy to the internal layout, no scratch
         CK(launch_restrict_canon(h->rp, g, h->blk[0], h->p.nvec[0], rp_vecs(h), fine, coarse, nrhs, st));
+        CK(cudaStreamSynchronize(st));   // the result is complete on return, whichever path the call takes
         return AMG_OK;
     }
     DevBuf tmp;
@@ -2929,6 +2930,7 @@ amg_status amg_prolong(amg_hierarchy* h, int coarsening, const void* coarse, voi
     int cprec = prec == AMG_F64 ? 0 : 1;
     if (prec == AMG_F32 && transfer_canon_supported(h->rp, cprec, fine) && transfer_apart(h, fine, coarse, nrhs)) {
         CK(launch_prolong_canon(h->rp, g, h->blk[0], h->p.nvec[0], rp_vecs(h), coarse, fine, nrhs, st));
+        CK(cudaStreamSynchronize(st));
         return AMG_OK;
     }
     DevBuf tmp;
