@@ -154,40 +154,47 @@ DEV void spin_mac(cx<float> acc[12], const cx<float>* w, const cx<float> phi[12]
         }
 }
 
-// |v|^2 as an unevaluated pair of floats: exact products, every rounding error kept, so that
-// the sums carry about 48 bits without the FP64 pipe (1/64 of the FP32 rate)
-DEV void add_square(dfloat& acc, float v) {
-    const float p = __fmul_rn(v, v);
-    const float e = fmaf(v, v, -p);
-    const dfloat t = two_sum(acc.hi, p);
-    acc.hi = t.hi;
-    acc.lo = __fadd_rn(acc.lo, __fadd_rn(t.lo, e));
-}
-
-// A thread's sum of squares of any FP32 values: a site whose largest component lies outside
-// [2^-50, 2^50] is scaled by a power of two first (FP32 squares would be lost or overflow) and its
-// sum goes to a double; the others' pairs add up as pairs
+// A thread's sum of squares of any FP32 values in FP64: a site's 24 squares on the FP32 pipe, with
+// the rounding errors of the products and of the sums kept so that nothing is lost that FP64 would
+// hold; the sites in FP64 (FP64 instructions run at 1/64 of the FP32 rate; a site takes six of
+// them instead of 48).
+// hi and mid start at powers of two c0 and c1 (times 1.5) that no term exceeds, so the three-operation
+// quick_two_sum is exact for them: squares are at most c0, the errors of hi and of the products at
+// most 2^-19 c0 and all 48 of them together below c1 / 2.  What lo loses is of order 2^-55 c0.
+// A site whose largest component lies outside [2^-38, 2^50] is scaled by a power of two first: the
+// errors of smaller squares would fall below the FP32 range, larger squares overflow it.
 struct SquareSum {
-    dfloat p;
     double d = 0;
     // the 24 components of a site, v(k)
     template <class F> DEV void add(F&& v) {
-        float m = 0.f, q = 0.f;
+        float m = 0.f;
 #pragma unroll
         for (int k = 0; k < 24; ++k) m = fmaxf(m, fabsf(v(k)));
-        const float sc = m < 0x1p-50f ? 0x1p100f : m > 0x1p50f ? 0x1p-100f : 1.f;
-        dfloat t;
+        const float sc = m < 0x1p-38f ? 0x1p80f : m > 0x1p50f ? 0x1p-80f : 1.f;
+        const float ms = sc * m;
+        const float c0 = __uint_as_float((__float_as_uint(ms * ms) & 0x7f800000u) + 0x00800000u);
+        const float c1 = 0x1.8p-12f * c0;
+        float hi = c0, mid = c1, lo = 0.f;
 #pragma unroll
         for (int k = 0; k < 24; ++k) {
-            const float x = sc * v(k);
-            add_square(t, x);
-            q = fmaf(x, x, q);
+            const float x = sc * v(k), p = __fmul_rn(x, x);
+            const dfloat t = quick_two_sum(hi, p), u = quick_two_sum(mid, t.lo);
+            const dfloat w = quick_two_sum(u.hi, fmaf(x, x, -p));
+            hi = t.hi;
+            mid = w.hi;
+            lo = __fadd_rn(lo, __fadd_rn(u.lo, w.lo));
         }
-        if (!(q <= 0x1.fffffep127f)) d += q;   // infinite or NaN: the pair would turn both into NaN
-        else if (sc == 1.f) p = p + quick_two_sum(t.hi, t.lo);
-        else d += to_double(t) * (sc > 1.f ? 0x1p-200 : 0x1p200);
+        if (!(fabsf(hi) <= 0x1.fffffep127f)) {   // an infinity or a NaN: the error terms would turn both into NaN
+            float q = 0.f;
+#pragma unroll
+            for (int k = 0; k < 24; ++k) q = fmaf(v(k), v(k), q);
+            d += q;
+            return;
+        }
+        const double t = ((double)lo + (double)__fsub_rn(mid, c1)) + (double)__fsub_rn(hi, c0);
+        d += sc == 1.f ? t : t * (sc > 1.f ? 0x1p-160 : 0x1p160);
     }
-    DEV double get() const { return to_double(p) + d; }
+    DEV double get() const { return d; }
 };
 
 // The last layer of a training pass: y is replaced by y - e for the canonical target e, and
