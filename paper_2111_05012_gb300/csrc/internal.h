@@ -60,11 +60,10 @@ struct amg_nn {
     DevBuf wadj[AMG_NN_MAX_LAYERS];         // bfloat16 adjoint weights (input gradient)
     DevBuf act[AMG_NN_MAX_LAYERS + 1];      // activations, FP32 internal fields x channels
     DevBuf gbuf[2];                         // gradient fields
-    DevBuf ework;                           // output field
+    DevBuf ework;                           // output field; in a training step an unaligned pair's target
     DevBuf part;                            // reduction partials
     DevBuf grad[AMG_NN_MAX_LAYERS];         // weight gradients, summed over a batch's pairs
     DevBuf norms;                           // per pair (|y - e|^2, |e|^2)
-    DevBuf ecopy;                           // aligned copy of an unaligned target batch
 };
 
 // accessors implemented in api.cu

@@ -204,22 +204,21 @@ amg_status amg_nn_train_step(amg_nn* nn, const float* r, const float* e, int npa
     cudaStream_t s = (cudaStream_t)stream;
     const GeomH& g = geom(nn);
     const int L = nn->nlayers;
-    if (((uintptr_t)e & 15) != 0) {
-        // the loss reads e in 16-byte words: an unaligned batch goes through an aligned copy
-        const size_t bytes = (size_t)npairs * g.V * 24 * sizeof(float);
-        NCK(nn->ecopy.ensure(bytes));
-        NCK(cudaMemcpyAsync(nn->ecopy.p, e, bytes, cudaMemcpyDeviceToDevice, s));
-        e = nn->ecopy.as<float>();
-    }
     NCK(nn->norms.ensure(npairs * sizeof(double2)));
     // every pair's gradient is summed on the device, scaled by 1 / |e|^2 as it is added; the
     // host waits once for the whole batch
     for (int p = 0; p < npairs; ++p) {
         double2* norm = nn->norms.as<double2>() + p;
+        const float* target = e + (size_t)p * g.V * 24;
+        if (((uintptr_t)target & 15) != 0) {
+            // the loss reads its target in 16-byte words: an unaligned one is copied, pair by pair
+            NCK(cudaMemcpyAsync(nn->ework.p, target, (size_t)g.V * 24 * sizeof(float), cudaMemcpyDeviceToDevice, s));
+            target = nn->ework.as<float>();
+        }
         NCK(launch_pack_spinor(1, g, r + (size_t)p * g.V * 24, nn->act[0].p, 1, s));
         for (int l = 0; l < L; ++l)
             NCK(launch_ptconv_forward(g, nn->ch[l], nn->ch[l + 1], amg_internal_links(nn->d, 1), nn->wbf[l].p,
-                                      nn->act[l].p, nn->act[l + 1].p, s, l == L - 1 ? e + (size_t)p * g.V * 24 : nullptr,
+                                      nn->act[l].p, nn->act[l + 1].p, s, l == L - 1 ? target : nullptr,
                                       nn->part.as<double2>(), norm));
         const void* gout = nn->act[L].p;   // y - e
         int gi = 0;
