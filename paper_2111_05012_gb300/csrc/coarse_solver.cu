@@ -642,19 +642,19 @@ __global__ void __launch_bounds__(kThreads) coarse_bicgstab_kernel(Args a) {
     coarse_bicgstab_body<TC, BF, NB>(a);
 }
 
-// several independent problems in one launch: cluster c (csize CTAs) solves problem c with
+// several independent problems (FP32 vectors) in one launch: cluster c (csize CTAs) solves problem c with
 // the arguments descs[c]; its barriers and reductions involve only its own CTAs
-template <typename TC, int BF>
+template <int BF>
 __global__ void __launch_bounds__(kThreads) coarse_bicgstab_multi_kernel(const Args* __restrict__ descs, int csize) {
     Args a = descs[blockIdx.x / csize];
     a.cta = blockIdx.x % csize;
     a.ncta = csize;
-    coarse_bicgstab_body<TC, BF, 1>(a);
+    coarse_bicgstab_body<float, BF, 1>(a);
 }
 
 // the same with a range of CTAs per problem (first .. first + ncta - 1) in one cooperative launch,
 // which keeps all of them resident for the problems' barriers
-template <typename TC, int BF>
+template <int BF>
 __global__ void __launch_bounds__(kThreads) coarse_bicgstab_split_kernel(const Args* __restrict__ descs, int np) {
     int lo = 0, hi = np - 1;
     while (lo < hi) {
@@ -664,7 +664,7 @@ __global__ void __launch_bounds__(kThreads) coarse_bicgstab_split_kernel(const A
     }
     Args a = descs[lo];
     a.cta = blockIdx.x - a.first;
-    coarse_bicgstab_body<TC, BF, 1>(a);
+    coarse_bicgstab_body<float, BF, 1>(a);
 }
 
 // one CTA per SM (152 barrier participants on GB300), if the kernel fits
@@ -796,6 +796,7 @@ cudaError_t launch_coarse_bicgstab_multi(const CoarseSolveDesc* d, int n, void* 
                                          cudaStream_t s) {
     if (n < 1) return cudaSuccess;
     const int cprec = d[0].cprec;
+    if (cprec != 1 && cprec != 2) return cudaErrorInvalidValue;   // batches are FP32 vectors
     Args* args = (Args*)host_args;
     int smem = 0;
     for (int i = 0; i < n; ++i) {
@@ -813,10 +814,8 @@ cudaError_t launch_coarse_bicgstab_multi(const CoarseSolveDesc* d, int n, void* 
     // waves, the large problems' the longest, up to 38; beyond that they keep the chip busy by
     // themselves.  12 problems of 8^4, 12^4 and 16^3 x 32: 1109 -> 477 us per solve of all.
     {
-        const void* fs = cprec == 0   ? (const void*)coarse_bicgstab_split_kernel<double, 0>
-                         : cprec == 3 ? (const void*)coarse_bicgstab_split_kernel<double, 2>
-                         : cprec == 1 ? (const void*)coarse_bicgstab_split_kernel<float, 0>
-                                      : (const void*)coarse_bicgstab_split_kernel<float, 1>;
+        const void* fs = cprec == 1 ? (const void*)coarse_bicgstab_split_kernel<0>
+                                    : (const void*)coarse_bicgstab_split_kernel<1>;
         cudaError_t e = cudaFuncSetAttribute(fs, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
         const int grid = coop_grid(fs, smem);
@@ -851,10 +850,8 @@ cudaError_t launch_coarse_bicgstab_multi(const CoarseSolveDesc* d, int n, void* 
     }
     cudaError_t e = cudaMemcpyAsync(dev_args, args, sizeof(Args) * n, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return e;
-    const void* fn = cprec == 0   ? (const void*)coarse_bicgstab_multi_kernel<double, 0>
-                     : cprec == 3 ? (const void*)coarse_bicgstab_multi_kernel<double, 2>
-                     : cprec == 1 ? (const void*)coarse_bicgstab_multi_kernel<float, 0>
-                                  : (const void*)coarse_bicgstab_multi_kernel<float, 1>;
+    const void* fn = cprec == 1 ? (const void*)coarse_bicgstab_multi_kernel<0>
+                                : (const void*)coarse_bicgstab_multi_kernel<1>;
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};

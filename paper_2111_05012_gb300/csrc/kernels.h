@@ -164,9 +164,10 @@ cudaError_t launch_coarse_bicgstab(int cprec, const GeomH& gc, int nc, const voi
                                    void* part, void* state, int cluster, cudaStream_t s, int nb = 1,
                                    int xgroup = 0);
 int coarse_solver_max_xgroup(int cprec, int nc, int nb);
-// several independent single-RHS solves in one launch, one thread-block cluster per problem
-// (each with its own vectors, operator, partials and state word); dev_args is device scratch of
-// n * coarse_solver_desc_bytes(); all problems share cprec
+// several independent single-RHS solves of FP32 vectors in one launch (each with its own vectors,
+// operator, partials and state word): up to a quarter of the SMs, a share of all SMs per problem by
+// the size of its operator, beyond that one thread-block cluster per problem; dev_args is device
+// scratch of n * coarse_solver_desc_bytes(); all problems share cprec (1 or 2)
 struct CoarseSolveDesc {
     int cprec;
     GeomH gc;
