@@ -114,7 +114,8 @@ cudaError_t launch_restrict_canon(int vprec, const GeomH& g, const BlockH& bk, i
                                   const void* fine, void* coarse, int nrhs, cudaStream_t s);
 cudaError_t launch_prolong_canon(int vprec, const GeomH& g, const BlockH& bk, int nvec, const void* vecs,
                                  const void* coarse, void* fine, int nrhs, cudaStream_t s);
-// block Gram-Schmidt (twice) in FP64 on nvec internal fine vectors; *err_flag set to 1 on rank deficiency
+// block Gram-Schmidt on nvec internal fine vectors, a second projection after a large cancellation
+// (FP64 vectors in FP64, FP32 vectors in float pairs); *err_flag set to 1 on rank deficiency
 cudaError_t launch_orthonormalise_fine(int vprec, const GeomH& g, const BlockH& bk, int nvec, void* vecs,
                                        int* err_flag, cudaStream_t s);
 // Galerkin coarse stencil from the fine operator; B layout [Vc][Nc][9][Nc] of cprec

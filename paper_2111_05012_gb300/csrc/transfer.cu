@@ -333,8 +333,9 @@ __global__ void prolong_ragged_kernel(const RaggedDev* __restrict__ d, const int
 // |w|^2: against an orthonormal set one projection leaves w orthogonal to about
 // eps |w0| / |w| <= 2 eps otherwise (the DGKS test).  Either way the result is
 // the QR factor with a positive diagonal to rounding, the vectors that
-// projecting one vector after another gives.
-// FP64 vectors; FP32 vectors take orthonormalise_pairs_kernel.
+// projecting one vector after another gives.  orthonormalise_kernel does this
+// for FP64 vectors, orthonormalise_pairs_kernel for FP32 vectors.
+
 // chirality half chi of a fine field at one site (plain loads: written earlier in the launch)
 template <class PV> DEV void load_chirality(const void* base, int V, int s, int chi, cx<typename PV::T> v[6]);
 template <> DEV void load_chirality<P32>(const void* base, int V, int s, int chi, cx<float> v[6]) {
@@ -363,7 +364,6 @@ __global__ void __launch_bounds__(512) orthonormalise_kernel(Geom g, Blocking bk
     const int l = threadIdx.x, lane = l & 31, warp = l >> 5, nw = blockDim.x >> 5;
     const bool active = l < bk.Vb;
     const size_t vb = spinor_bytes<P64>(g.V);
-    constexpr int G = 1;   // previous vectors in flight (more spill at the 128 registers of 512 threads)
     int c[4], s = 0;
     if (active) s = block_site(g, bk, Xi, l, c);
     auto load_half = [&](int j, cx<double> (&q)[6]) {
@@ -390,28 +390,18 @@ __global__ void __launch_bounds__(512) orthonormalise_kernel(Geom g, Blocking bk
                 block_sum<double, 1>(n1, red);
                 if (n1[0] > 0.25 * n0[0]) break;
             }
-            // G previous vectors at a time: their loads in flight together, and their sums taken over
-            // the warp by transposed shuffles (10 FP64 additions for four sums instead of 20)
-            for (int j0 = 0; j0 < i; j0 += G) {
-                cx<double> u[G][6];
+            for (int j = 0; j < i; ++j) {
+                cx<double> d = czero<double>();
+                if (active) {
+                    cx<double> u[6];
+                    load_chirality<P64>((const char*)vecs + j * vb, g.V, s, chi, u);
 #pragma unroll
-                for (int t = 0; t < G; ++t)
-                    if (active && j0 + t < i) load_chirality<P64>((const char*)vecs + (j0 + t) * vb, g.V, s, chi, u[t]);
-                double q[2 * G];
-#pragma unroll
-                for (int t = 0; t < G; ++t) {
-                    cx<double> d = czero<double>();
-                    if (active && j0 + t < i) {
-#pragma unroll
-                        for (int k = 0; k < 6; ++k) cfmac(d, u[t][k], w[k]);
-                    }
-                    q[2 * t] = d.re;
-                    q[2 * t + 1] = d.im;
+                    for (int k = 0; k < 6; ++k) cfmac(d, u[k], w[k]);
                 }
-                const double tot = transposed_warp_sum<2 * G>(q, lane);
-                const int v = transposed_index<2 * G>(lane);
-                if ((lane & (32 / (2 * G) - 1)) == 0 && j0 + (v >> 1) < i)
-                    reinterpret_cast<double*>(part + warp * nvec + j0 + (v >> 1))[v & 1] = tot;
+                // the upper half of the warp ends with the sum of the imaginary parts
+                double q[2] = {d.re, d.im};
+                const double tot = transposed_warp_sum<2>(q, lane);
+                if ((lane & 15) == 0) reinterpret_cast<double*>(part + warp * nvec + j)[lane >> 4] = tot;
             }
             __syncthreads();
             for (int j = l; j < i; j += blockDim.x) {
@@ -420,18 +410,12 @@ __global__ void __launch_bounds__(512) orthonormalise_kernel(Geom g, Blocking bk
                 coef[j] = t;
             }
             __syncthreads();
-            for (int j0 = 0; j0 < i; j0 += G) {
-                cx<double> u[G][6];
+            for (int j = 0; j < i && active; ++j) {
+                cx<double> u[6];
+                load_chirality<P64>((const char*)vecs + j * vb, g.V, s, chi, u);
+                const cx<double> cc = -coef[j];
 #pragma unroll
-                for (int t = 0; t < G; ++t)
-                    if (active && j0 + t < i) load_chirality<P64>((const char*)vecs + (j0 + t) * vb, g.V, s, chi, u[t]);
-#pragma unroll
-                for (int t = 0; t < G; ++t) {
-                    if (!active || j0 + t >= i) break;
-                    const cx<double> cc = -coef[j0 + t];
-#pragma unroll
-                    for (int k = 0; k < 6; ++k) cfma(w[k], cc, u[t][k]);
-                }
+                for (int k = 0; k < 6; ++k) cfma(w[k], cc, u[k]);
             }
             __syncthreads();   // part / coef are rewritten by the next pass
         }
