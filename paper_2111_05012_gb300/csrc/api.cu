@@ -379,7 +379,7 @@ amg_status fine_sap(amg_hierarchy* h, int prec, const void* b, void* x, bool x_z
     amg_dirac* d = h->d;
     h->timer.start(PH_SMOOTH, s);
     // sap_variant 3: the FP16 copy of the operator under FP32 vectors
-    const bool op16 = h->p.sap_variant == 3 && prec == 1 && sap_staged_supported(1, h->blk[0]);
+    const bool op16 = h->p.sap_variant == 3 && prec == 1 && sap_pairs_supported(1, h->blk[0]);
     for (int i = 0; i < h->p.sap_iters; ++i) {
         const bool first = x_zero && i == 0;
         for (int colour = 0; colour < 2; ++colour) {

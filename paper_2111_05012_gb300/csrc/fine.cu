@@ -2342,7 +2342,7 @@ cudaError_t launch_clover_invert(int prec, const GeomH& gh, const void* C64, voi
 
 cudaError_t launch_sap_half(int prec, const GeomH& g, const BlockH& bk, int colour, int nmr, int x_mode, const void* U,
                             const void* C, const void* b, void* x, double kappa, int nrhs, cudaStream_t st) {
-    if (sap_staged_supported(prec, bk))
+    if (sap_pairs_supported(prec, bk))
         return prec == 1 ? sap_pairs_impl<P32>(g, bk, colour, nmr, x_mode, U, C, b, x, kappa, nrhs, st)
                          : sap_pairs_impl<P16>(g, bk, colour, nmr, x_mode, U, C, b, x, kappa, nrhs, st);
     if (prec == 0) return sap_half_impl<P64>(g, bk, colour, nmr, x_mode, U, C, b, x, kappa, nrhs, st);
@@ -2354,7 +2354,7 @@ cudaError_t launch_sap_half_staged16(const GeomH& g, const BlockH& bk, int colou
                                      const void* b, void* x, double kappa, int nrhs, cudaStream_t st) {
     return sap_half_staged_impl<P32, P16>(g, bk, colour, nmr, x_mode, U32, C32, b, x, kappa, nrhs, st, U16, C16);
 }
-bool sap_staged_supported(int prec, const BlockH& bk) {
+bool sap_pairs_supported(int prec, const BlockH& bk) {
     int vb = bk.b[0] * bk.b[1] * bk.b[2] * bk.b[3];
     return (prec == 1 || prec == 2) && vb <= 256;
 }

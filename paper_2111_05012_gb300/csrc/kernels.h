@@ -85,7 +85,7 @@ cudaError_t launch_sap_half(int prec, const GeomH& g, const BlockH& bk, int colo
                             const void* U, const void* C, const void* b, void* x, double kappa, int nrhs,
                             cudaStream_t s);
 // FP32 / FP16 domains of at most 256 sites (packed-pair kernel; staged FP16 operator for FP32)
-bool sap_staged_supported(int prec, const BlockH& bk);
+bool sap_pairs_supported(int prec, const BlockH& bk);
 // variant 3 (FP32 smoother, blocks <= 256 sites): the domain operator staged in shared memory from
 // its FP16 copy (U16, C16: prec-2 fields), FP32 arithmetic and vectors; the residual b - D x uses
 // the FP32 operator
