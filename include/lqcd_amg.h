@@ -240,25 +240,27 @@ amg_status amg_dirac_get_clover(amg_dirac* d, double* host_out);
  * double out for AMG_F64X.  in and out must not alias. */
 amg_status amg_apply_D(amg_dirac* d, const void* in, void* out, int nrhs, amg_prec prec, amg_stream s);
 
-/* out = D in, exactly as amg_apply_D, but without allocating device memory.
+/* out = D in, as amg_apply_D (to rounding), but without allocating device memory.
  * The paper has no counterpart: this entry point exists for callers that
  * cannot allocate, e.g. a process whose device memory is fully reserved by a
  * caching allocator or a latency-critical loop that must not pay the
  * device-wide synchronisation of cudaMalloc/cudaFree.  amg_apply_D converts
- * the canonical vectors to and from the internal layout in two work fields
- * the library allocates on first use; this variant keeps those two fields in
- * one static device array of 24 MiB (12 MiB each) that every GPU loading the
- * library holds until exit.  The first call on a device looks up the array's
- * device address (cudaGetSymbolAddress) once for that device and keeps it for
- * the life of the process; make that first call before any stream capture.
- * Resetting the device (cudaDeviceReset) or otherwise recreating its primary
- * context after that first call is not supported: the array may then live at
- * another address.  Every call shares the array, so calls that
- * overlap on the GPU (different streams, or host threads) race: serialise
- * them.  nrhs * fine_field_bytes(prec) must be <= 12 MiB, where a field is
- * 192 (AMG_F64), 96 (AMG_F32) or 52 (AMG_F16) bytes per site; larger calls
- * fail with AMG_EINVAL.  in, out: canonical device vectors as for
- * amg_apply_D (element type double for AMG_F64, float otherwise). */
+ * half-precision inputs, and vectors that are not 16-byte aligned or that
+ * overlap, to and from the internal layout in work fields the library
+ * allocates on first use; this variant converts every call's vectors, in two
+ * fields kept in one static device array of 24 MiB (12 MiB each) that every
+ * GPU loading the library holds until exit.  The first call on a device looks
+ * up the array's device address (cudaGetSymbolAddress) once for that device
+ * and keeps it for the life of the process; make that first call before any
+ * stream capture.  Resetting the device (cudaDeviceReset) or otherwise
+ * recreating its primary context after that first call is not supported: the
+ * array may then live at another address.  Every call shares the array, so
+ * calls that overlap on the GPU (different streams, or host threads) race:
+ * serialise them.  nrhs * fine_field_bytes(prec) must be <= 12 MiB, where a
+ * field is 192 (AMG_F64), 96 (AMG_F32) or 52 (AMG_F16; the field rounded up to
+ * whole 16-byte words) bytes per site; larger calls fail with AMG_EINVAL.
+ * in, out: canonical device vectors as for amg_apply_D (element type double
+ * for AMG_F64, float otherwise). */
 amg_status amg_apply_D_noalloc(amg_dirac* d, const void* in, void* out, int nrhs, amg_prec prec, amg_stream s);
 
 /* Autotune the launch shape of the fine stencil in precision prec (AMG_F64,
@@ -266,9 +268,10 @@ amg_status amg_apply_D_noalloc(amg_dirac* d, const void* in, void* out, int nrhs
  * the register budget (2 resident CTAs per SM, 128 registers, against the
  * default).  The choice is process-wide and used by every later stencil
  * launch of that precision (amg_setup runs the same tuner for the precisions
- * a solve uses); amg_apply_D on 16-byte aligned vectors runs a kernel of its own
- * on the canonical layout, in a fixed shape.  Outputs (may be NULL): threads per CTA, grid cap in CTAs
- * per SM, register budget as resident CTAs per SM (0 = the default).
+ * a solve uses); amg_apply_D on 16-byte aligned vectors runs a kernel of its
+ * own on the canonical layout, in a fixed shape.  Outputs (may be NULL):
+ * threads per CTA, grid cap in CTAs per SM, register budget as resident CTAs
+ * per SM (0 = the default).
  * Synchronises the device.  No counterpart in the paper. */
 amg_status amg_dirac_tune(amg_dirac* d, amg_prec prec, int* threads, int* per_sm, int* regs_ctas);
 
@@ -298,10 +301,12 @@ amg_status amg_apply_Dsap(amg_dirac* d, const int block[4], const void* in, void
 /* ---- multigrid hierarchy (Sec. 3 step 0) ------------------------------ */
 
 /* Adaptive setup, steps (0-a) and (0-b) of Sec. 3: the init vectors are
- * smoothed by n_init SAP applications, block-orthonormalised in FP64 per
- * (domain, chirality) by Gram-Schmidt applied twice, the Galerkin coarse
- * operator D_c = <I|D|J> (Eq. 7) is built, then n_adapt passes v <- M v
- * follow.  init_vecs[l] is a host array of nvec[l] canonical vectors of
+ * smoothed by n_init SAP applications, block-orthonormalised per (domain,
+ * chirality) by Gram-Schmidt with a second projection where the first removed
+ * most of a vector (FP64 vectors in FP64; FP32 vectors in pairs of floats, 48
+ * bits, and rounded to FP32 at the end), the Galerkin coarse operator
+ * D_c = <I|D|J> (Eq. 7) is built, then n_adapt passes v <- M v follow.
+ * init_vecs[l] is a host array of nvec[l] canonical vectors of
  * level l (doubles: fine [site][spin][colour][re, im], coarse
  * [site][Nc][re, im]), one array for every level 0..nlevels-2, each in host
  * or device memory (copied with cudaMemcpyDefault); the random numbers of
@@ -400,13 +405,17 @@ amg_status amg_precondition(amg_hierarchy* h, const double* b, double* x, amg_st
  * smoother, FP32 coarse vectors, the same coarse operator storage, test-vector
  * precision, sap_iters and mr_iters, blocks of at most 256 sites and
  * outer_m <= 19): each phase of an Arnoldi step -- the FP64 -> FP32 copy of
- * V_j, restriction, the coarse BiCGStab(l) (one thread-block cluster per
- * problem), prolongation, each SAP half sweep, the Arnoldi product and the
- * Gram-Schmidt pass -- is one kernel launch over a table of per-problem
- * descriptors, whatever n is.  Otherwise (or after amg_set_ragged_fusion(0))
+ * V_j, restriction, the coarse BiCGStab(l) (a share of all SMs per problem, by
+ * the size of its operator, for up to a quarter as many active problems as
+ * SMs; beyond that one thread-block cluster per problem), prolongation, each
+ * SAP half sweep, the Arnoldi product and the Gram-Schmidt pass -- is one
+ * kernel launch over a table of per-problem descriptors, whatever n is.  Otherwise (or after amg_set_ragged_fusion(0))
  * each problem's step runs on a pool of up to 16 streams, captured into a
  * CUDA graph on first use (kept in the hierarchy until its workspaces grow
- * or its learned correction changes) and replayed.  b[i], x[i]: canonical
+ * or its learned correction changes) and replayed.  In the fused form the order
+ * of a problem's coarse sums follows its share of the SMs, so the last bits of
+ * its FP32 preconditioner depend on the other problems of the batch and on when
+ * they converge; the FP64 tolerance does not.  b[i], x[i]: canonical
  * double device vectors of problem i.  infos (may be NULL) receives n
  * records.  Ordered after earlier work on stream s; synchronises.  No
  * counterpart in the paper (a batch of independent solves of Sec. 3). */

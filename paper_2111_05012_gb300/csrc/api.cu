@@ -1933,7 +1933,7 @@ amg_status fgmres_ragged(std::vector<RaggedProb>& P, const std::vector<cudaStrea
 // (ragged_dev_fill) and per-phase prefix tables of CTA offsets split each grid
 // among the problems, so a problem of 4^4 sites and one of 16^3 x 32 share a
 // launch.  Per step: FP64 -> FP32 copy of V_j, restriction, the coarse
-// BiCGStab(l) (one thread-block cluster per problem in one launch), prolongation,
+// BiCGStab(l) (a share of the SMs or a cluster per problem, in one launch), prolongation,
 // 2 sap_iters SAP half sweeps, the FP64-accurate Arnoldi product and a
 // classical Gram-Schmidt pass -- 2 sap_iters + 8 kernels for the whole batch,
 // whatever its size.  Used when every problem has an FP32 smoother, FP32
