@@ -954,7 +954,7 @@ def run_coarse_tc(args):
             # traffic: dram__bytes_read.sum + dram__bytes_write.sum of one coarse_tc_kernel<32> launch (16 RHS)
             # on this workload from an ncu --set full capture (708.8 + 47.6 MB)
             "roofline": {"kernel": "coarse_tc_kernel<32>", "bound": "hbm", "achieved": t["gb_per_s"], "peak": hbm,
-                         "unit": "GB/s", "frac": t["frac_hbm"], "traffic": 756.4e6, "peak_kind": kind},
+                         "unit": "GB/s", "frac": t["frac_hbm"], "traffic": 758.2e6, "peak_kind": kind},
             "gpu_launches": t["launches"], "clocks": clk.summary()}
     capi.amg_hierarchy_destroy(h)
     capi.amg_dirac_destroy(d)
