@@ -952,7 +952,7 @@ def run_coarse_tc(args):
                        "coarse_sites": Vc, "nc": nc, "l2": "operator image 680 MB > L2 (no flush)",
                        "variants": res},
             # traffic: dram__bytes_read.sum + dram__bytes_write.sum of one coarse_tc_kernel<32> launch (16 RHS)
-            # on this workload from an ncu --set full capture (708.8 + 47.6 MB)
+            # on this workload from an ncu capture (709.4 + 48.8 MB)
             "roofline": {"kernel": "coarse_tc_kernel<32>", "bound": "hbm", "achieved": t["gb_per_s"], "peak": hbm,
                          "unit": "GB/s", "frac": t["frac_hbm"], "traffic": 758.2e6, "peak_kind": kind},
             "gpu_launches": t["launches"], "clocks": clk.summary()}
